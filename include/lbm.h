@@ -155,8 +155,10 @@ int lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_
 int lbm_init_fields(lbm_handle* h, const double* phi, const double* psi, const double* ux,
                     const double* uy, const double* P, int mem);
 
-/* Advance n >= 0 time steps: one fused collide-stream kernel launch per step (pull streaming,
- * stencils on halo tiles in shared memory, moment-space collision of f, g and h).
+/* Advance n >= 0 time steps (pull streaming, stencils on halo tiles in shared memory, moment-space
+ * collision of f, g and h, fused in one kernel).  Unless lbm_set_kernel chose a kernel, many steps go
+ * in one launch, whose tiles wait for their neighbours of the step before (at least 4 or 8 steps,
+ * depending on the grid); fewer steps are one launch each.  The state is the same bit for bit.
  * Asynchronous: errors found by the device surface at the next synchronous call. */
 int lbm_step(lbm_handle* h, int64_t n);
 
@@ -230,7 +232,7 @@ int lbm_steps_taken(const lbm_handle* h, int64_t* steps);
 /* Free the handle (not the workspace).  Waits for the handle's stream.  NULL is allowed. */
 int lbm_destroy(lbm_handle* h);
 
-/* Step kernel of a handle.  Both variants compute the same step bit for bit; they differ in how
+/* Kernel of a single step of a handle.  Both variants compute the same step bit for bit; they differ in how
  * the work is laid out on the GPU (FP32 storage: one cell per thread, tiles of 32 x 8 cells;
  * 16-bit storage: two horizontally adjacent cells per thread, tiles of 32 x 8 cells):
  *   LBM_KERNEL_TILE       one CTA per tile, launched as a grid of all tiles;
@@ -240,7 +242,9 @@ int lbm_destroy(lbm_handle* h);
  *   LBM_KERNEL_AUTO       (lbm_set_kernel only) the library's choice, the faster one on GB300
  *                         at 2048 x 1024 cells: PIPELINED for 16-bit storage and for a density
  *                         ratio != 1, TILE for FP32 storage at uniform density.
- * A new handle uses the library's choice.  LBM_EINVAL if the pipelined kernel does not fit. */
+ * A new handle uses the library's choice, and takes runs of steps in one launch (lbm_step); with
+ * TILE or PIPELINED set, every step is one launch of that kernel.  LBM_EINVAL if the pipelined kernel
+ * does not fit. */
 #define LBM_KERNEL_AUTO 0
 #define LBM_KERNEL_TILE 1
 #define LBM_KERNEL_PIPELINED 2

@@ -4,6 +4,7 @@
 //   [pops A | pops B | u history A | u history B | (S history A | S history B) | status word | reduction partials]
 // every part 256-byte aligned.  Between steps the population buffer that is not current is dead
 // (the next step overwrites all of it), so host transfers stage through it.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -291,6 +292,94 @@ int launch_step(lbm_handle* h, int mode, double* const out[5]) {
     return LBM_OK;
 }
 
+// Counters of a run of steps: the tile counter, then the row counters.  They share the reduction's
+// partial sums (work of one handle is ordered on its stream).
+constexpr int kRowOffset = 32, kRowCounters = 2016;
+static_assert((kRowOffset + kRowCounters) * sizeof(unsigned) <= lbm::kMaxPartials * sizeof(double),
+              "the counters fit the partial sums");
+
+// Whether `n` steps in a row go as runs (one launch for many steps).  Always the faster way but for a
+// few steps, whose launch and counters' reset cost more than they save (at 128 x 128: 4.3 us per step
+// one by one, 4.0 in a run, 5 us once per run), and for 16-bit grids of one to three tiles per SM,
+// where all tiles are resident at once either way and the one-tile kernel hands over faster (FP16
+// 300 x 300: 5.6 us, a run 7.0; 128 x 128: 5.1 / 4.8; 500 x 300: 7.9 / 7.0).
+bool takes_run(const lbm_handle* h, int64_t n) {
+    const long long tiles = (long long)h->tiles_x * h->tiles_y;
+    if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || tiles > 1 << 24) return false;
+    if (n < (tiles > 8 * h->sms ? 4 : 8)) return false;
+    return !(lbm::pair_is_16bit(h->prm.storage) && tiles > h->sms && tiles <= 3 * h->sms);
+}
+
+// Launch a run of at most n steps; *took receives their number.
+int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
+    lbm::RunArgs a;
+    std::memset(&a, 0, sizeof(a));
+    for (int b = 0; b < 2; ++b) {
+        a.tm_fg[b] = h->tm_fg[b];
+        a.tm_h[b] = h->tm_h[b];
+        a.tm_hist[b] = h->tm_hist[b];
+        a.pops[b] = h->pops[b];
+        a.hist[b] = h->hist[b];
+        a.shist[b] = h->shist[b];
+    }
+    a.p = h->phys;
+    a.status = h->status;
+    a.steps = h->steps;
+    a.cur = h->cur;
+    a.first = h->first;
+    a.ntx = h->tiles_x;
+    a.nty = h->tiles_y;
+    const long long tiles = (long long)a.ntx * a.nty;
+    // launches of some tens of milliseconds at most, and positions within 32 bits
+    const int64_t most = std::max<int64_t>(64, (1LL << 20) / tiles);
+    *took = a.nsteps = (int)std::min(n, most);
+    // A tile reads two rows of cells above and below; only a last tile row of one cell row, next to the
+    // first around a periodic edge, makes that two tile rows.
+    const lbm::TileDims td = lbm::tile_dims(h->prm.storage);
+    a.reach = h->prm.bc_y == LBM_BC_PERIODIC && h->prm.ny % td.ty == 1 ? 2 : 1;
+    const int slots = h->sms * h->run.blocks_per_sm;
+    a.ring = h->run.buffers;
+    a.ahead = 16;
+    a.depth = 1;
+    a.lag = 1;
+    const bool pair16 = lbm::pair_is_16bit(h->prm.storage);
+    // Updating a row several times while it is in L2 pays for FP32 storage beyond L2 (129 MB), whose
+    // step is bound by HBM, where the rows in flight leave room for it: `lag` rows between levels must
+    // hold twice the tiles staged at a time, or tiles wait for the level before, and the band of
+    // depth x lag rows has to stay in L2 (us per step, one level at a time / so: sheared drop
+    // 2048 x 1024 68.8 / 67.1, 2048^2 136.5 / 132.5, rising bubble 1024 x 2048 76.7 / 72.8; FP16
+    // sheared drop 43.3 / 49.0).
+    const double cell_bytes = 2.0 * (lbm::pop_bytes_per_cell(h->prm.storage, h->prm.velocity == LBM_VELOCITY_SOLVED) +
+                                     sizeof(float2) * (h->shist[0] ? 2 : 1));
+    const double row_bytes = cell_bytes * h->L.pitch * td.ty;
+    if (!pair16 && row_bytes * a.nty > 160e6) {
+        for (int depth = 4; depth >= 3; --depth) {
+            const int lag = std::max(2 * a.reach, 1 + (2 * slots * a.ring + depth * a.ntx - 1) / (depth * a.ntx));
+            if (depth * lag * row_bytes <= 104e6 && a.nty >= 3 * depth * lag && a.nsteps >= depth) {
+                a.depth = depth;
+                a.lag = lag;
+                break;
+            }
+        }
+    }
+    // Claimed tiles balance the SMs, whose shares of the memory differ (2048 x 1024, one level at a
+    // time, fixed / claimed: FP32 78.3 / 68.8, FP16 47.0 / 43.3); a claim takes four, since the lead
+    // warp's round takes 2 us.  Up to about ten tiles per SM fixed positions do better (608 x 512 FP32
+    // 8.3 / 8.7, 128 x 128 4.0 / 5.2), and so do several levels at a time, which claims ahead of their
+    // turn would hold apart (67.1 / 69.4).
+    const bool fixed = a.depth > 1 || tiles <= 10LL * slots;
+    a.batch = !fixed ? 4 : (tiles <= 4LL * slots ? 1 : 2);
+    const int ctas = (int)std::min<long long>(tiles, slots);
+    unsigned* c = reinterpret_cast<unsigned*>(h->partials);
+    LBM_CUDA(cudaMemsetAsync(c, 0, (size_t)(kRowOffset + a.nty) * sizeof(unsigned), h->stream));
+    a.ctr = fixed ? nullptr : c;
+    a.rows = c + kRowOffset;
+    h->last_pipe_step = -2;
+    cudaError_t e = lbm::launch_run(h->prm.storage, a, variant_of(h->prm, h->phys.var_rho != 0), ctas, h->stream);
+    if (e != cudaSuccess) return fail(LBM_ECUDA, "run launch: %s", cudaGetErrorString(e));
+    return LBM_OK;
+}
+
 // FP64 sum of phi (lane 0) or psi (lane 1) of a population buffer into partials[0..blocks),
 // then partials[blocks] ... written to *dres.
 int launch_reduce(int st, const void* pops, int lane, bool pulled, int nx, int ny, int pitch, size_t plane, long long org,
@@ -477,9 +566,11 @@ int lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_
     h->tile_ctr = h->status + 2;
     h->last_pipe_step = -2;
     h->partials = reinterpret_cast<double*>(h->ws + L.off_partials);
-    int bps = 0, bps_pipe = 0, sms = 0;
+    int bps = 0, bps_pipe = 0;
     rc = prepare_kernels(p->storage, variant_of(*p, h->phys.var_rho != 0), &bps, &bps_pipe);
-    if (!rc && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess)
+    if (!rc && lbm::prepare_run(p->storage, variant_of(*p, h->phys.var_rho != 0), &h->run) != cudaSuccess)
+        rc = fail(LBM_ECUDA, "kernel setup failed");
+    if (!rc && cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess)
         rc = fail(LBM_ECUDA, "cudaDeviceGetAttribute failed");
     const bool pair16 = lbm::pair_is_16bit(p->storage), h16 = lbm::h_is_16bit(p->storage);
     const lbm::TileDims td = lbm::tile_dims(p->storage);
@@ -508,7 +599,7 @@ int lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_
     h->tiles_x = (p->nx + td.tx - 1) / td.tx;
     h->tiles_y = (p->ny + td.ty - 1) / td.ty;
     {
-        const long long ntiles = (long long)h->tiles_x * h->tiles_y, slots = (long long)bps_pipe * sms;
+        const long long ntiles = (long long)h->tiles_x * h->tiles_y, slots = (long long)bps_pipe * h->sms;
         h->pipe_ctas = (int)(ntiles < slots ? ntiles : slots);
         h->kernel = default_kernel(p->storage, variant_of(*p, h->phys.var_rho != 0), bps_pipe);
     }
@@ -586,12 +677,14 @@ int lbm_step(lbm_handle* h, int64_t n) {
     if (!h) return fail(LBM_EINVAL, "handle is NULL");
     if (!h->initialized) return fail(LBM_ESTATE, "lbm_step before lbm_init_fields");
     if (n < 0) return fail(LBM_EINVAL, "negative step count");
-    for (int64_t k = 0; k < n; ++k) {
-        int rc = launch_step(h, lbm::kStep, nullptr);
+    while (n > 0) {
+        int64_t took = 1;
+        int rc = takes_run(h, n) ? launch_run(h, n, &took) : launch_step(h, lbm::kStep, nullptr);
         if (rc) return rc;
-        h->cur ^= 1;
+        h->cur = (int)((h->cur + took) & 1);
         h->first = 0;
-        h->steps++;
+        h->steps += took;
+        n -= took;
     }
     return LBM_OK;
 }
@@ -743,12 +836,14 @@ int lbm_set_kernel(lbm_handle* h, int variant) {
         int rc = prepare_kernels(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0), &bps, &bps_pipe);
         if (rc) return rc;
         h->kernel = default_kernel(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0), bps_pipe);
+        h->chosen = 0;
         return LBM_OK;
     }
     if (variant != LBM_KERNEL_TILE && variant != LBM_KERNEL_PIPELINED) return fail(LBM_EINVAL, "bad kernel variant");
     if (variant == LBM_KERNEL_PIPELINED && h->pipe_ctas < 1)
         return fail(LBM_EINVAL, "the pipelined kernel does not fit on an SM for this storage mode");
     h->kernel = variant;
+    h->chosen = 1;
     return LBM_OK;
 }
 

@@ -236,10 +236,11 @@ template <int ST> struct Smem {
     static constexpr int H_SLOT = round128(H_BOX * H_ES);
     static constexpr int HIST_W = kHalo ? G::BW : G::TX, HIST_H = kHalo ? G::BH : G::TY;
     static constexpr int HIST_BYTES = HIST_W * HIST_H * 8;
+    // (f, g) boxes, u history, h boxes (last: a prescribed velocity stages none)
     static constexpr int FG = 0;
-    static constexpr int H = FG + kPairs * FG_SLOT;
-    static constexpr int HIST = H + H_SLOTS * H_SLOT;
-    static constexpr int PP = HIST + round128(HIST_BYTES);
+    static constexpr int HIST = FG + kPairs * FG_SLOT;
+    static constexpr int H = HIST + round128(HIST_BYTES);
+    static constexpr int PP = H + H_SLOTS * H_SLOT;
     static constexpr int PP_BYTES = round128(G::NE * 8);
     static constexpr int BAR = PP + PP_BYTES;
     static constexpr int BYTES = BAR + 16;
@@ -534,17 +535,29 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32
 __device__ __forceinline__ void mbar_arrive(unsigned long long* m) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(m)) : "memory");
 }
-// Named barrier 1 of the N compute threads of a warp-specialised CTA (its copy warp never takes
-// part); the OR form also tells every thread whether any of them passed true.
-template <int N> __device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(N) : "memory"); }
-template <int N> __device__ __forceinline__ bool compute_sync_or(bool v) {
+// Named barrier `id` of the N compute threads of one group of a warp-specialised CTA (its other
+// warps never take part); the OR form also tells every thread whether any of them passed true.
+template <int N> __device__ __forceinline__ void compute_sync(int id) {
+    asm volatile("bar.sync %0, %1;\n" ::"r"(id), "n"(N) : "memory");
+}
+template <int N> __device__ __forceinline__ bool compute_sync_or(int id, bool v) {
     uint32_t r;
     asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, 1, %2, q;\n selp.u32 %0, 1, 0, p;\n}\n"
+        "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, %3, %2, q;\n selp.u32 %0, 1, 0, p;\n}\n"
         : "=r"(r)
-        : "r"((uint32_t)v), "n"(N)
+        : "r"((uint32_t)v), "n"(N), "r"(id)
         : "memory");
     return r != 0;
+}
+// Whether a phase of the mbarrier is complete (no wait).
+__device__ __forceinline__ bool mbar_test(unsigned long long* m, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred P1;\n mbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n selp.u32 %0, 1, 0, P1;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(m)), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, int c0, int c1, int c2,
                                             unsigned long long* m) {
@@ -670,23 +683,30 @@ __device__ __forceinline__ Stencil stencil9(float2 C_, float2 E, float2 W, float
     return s;
 }
 
-// Stage the boxes of tile (x0, y0) with TMA on one mbarrier (called by one thread).
+// Stage boxes FIRST, FIRST + STRIDE, .. of tile (x0, y0) with TMA on one mbarrier (called by one thread).
+template <int ST, int FLOW, int FIRST = 0, int STRIDE = 1>
+__device__ __forceinline__ void issue_boxes(unsigned char* sm, const CUtensorMap* tm_fg, const CUtensorMap* tm_h,
+                                            const CUtensorMap* tm_hist, int x0, int y0, unsigned long long* mbar) {
+    using T = Traits<ST>;
+    using S = Smem<ST>;
+    constexpr int NH = FLOW ? S::H_SLOTS : 0;
+#pragma unroll
+    for (int n = FIRST; n < kPairs + NH + 1; n += STRIDE) {
+        if (n < kPairs)
+            tma_load_3d(sm + S::FG + n * S::FG_SLOT, tm_fg, x0 - 4 + kGX, y0 - 1 - cy(n) + kGY, n, mbar);
+        else if (n < kPairs + NH)
+            tma_load_3d(sm + S::H + (n - kPairs) * S::H_SLOT, tm_h, x0 - T::H_X0 + kGX, y0 + h_row0(n - kPairs) + kGY,
+                        n - kPairs, mbar);
+        else if (S::kHalo) tma_load_3d(sm + S::HIST, tm_hist, x0 - 4 + kGX, y0 - 1 + kGY, 0, mbar);
+        else tma_load_3d(sm + S::HIST, tm_hist, x0 + kGX, y0 + kGY, 0, mbar);
+    }
+}
+// Stage all boxes of tile (x0, y0) with TMA on one mbarrier (called by one thread).
 template <int ST, int FLOW>
 __device__ __forceinline__ void issue_tile_loads(unsigned char* sm, const CUtensorMap* tm_fg, const CUtensorMap* tm_h,
                                                  const CUtensorMap* tm_hist, int x0, int y0, unsigned long long* mbar) {
-    using T = Traits<ST>;
-    using S = Smem<ST>;
-    mbar_expect_tx(mbar, FLOW ? S::TX_BYTES : S::TX_BYTES_NOH);
-#pragma unroll
-    for (int i = 0; i < kPairs; ++i)
-        tma_load_3d(sm + S::FG + i * S::FG_SLOT, tm_fg, x0 - 4 + kGX, y0 - 1 - cy(i) + kGY, i, mbar);
-    if constexpr (FLOW) {
-#pragma unroll
-        for (int j = 0; j < S::H_SLOTS; ++j)
-            tma_load_3d(sm + S::H + j * S::H_SLOT, tm_h, x0 - T::H_X0 + kGX, y0 + h_row0(j) + kGY, j, mbar);
-    }
-    if constexpr (S::kHalo) tma_load_3d(sm + S::HIST, tm_hist, x0 - 4 + kGX, y0 - 1 + kGY, 0, mbar);
-    else tma_load_3d(sm + S::HIST, tm_hist, x0 + kGX, y0 + kGY, 0, mbar);
+    mbar_expect_tx(mbar, FLOW ? Smem<ST>::TX_BYTES : Smem<ST>::TX_BYTES_NOH);
+    issue_boxes<ST, FLOW>(sm, tm_fg, tm_h, tm_hist, x0, y0, mbar);
 }
 
 // Flow population I of the thread's cells, pulled from the staged h boxes.  16-bit h: plus the
@@ -770,14 +790,16 @@ __device__ __forceinline__ C load_h(const unsigned char* sm, const float2* Hist,
 // a one-cell ring give (phi, psi) for the 9-point stencils; the same boxes hold the own cell's
 // unshifted post-collision values, whose sums are phi and psi of the previous level
 // (m*_0 = phi exactly, Sec. 3.1), so only u of the previous level is stored.
-// WS: called by the compute warps of a warp-specialised CTA, which synchronise among themselves
-// with named barrier 1 only (the copy warp has staged the tile and waits on its own barriers).
+// WS: called by the NT threads of one compute group of a warp-specialised CTA, which synchronise
+// among themselves with named barrier `bar` only; t is the thread's index in the group, and `late`
+// tells that the caller's own wait for the tile already gave up.
 // EDGE = false: the tile is interior (tile_is_interior): every cell and every ring cell lies in
 // the grid away from its edges, so no cell writes ghost-frame copies, meets a wall or lies beyond
 // the grid, and those tests compile away.  The arithmetic is the same on both paths.
 template <int ST, bool WALLS, bool LANGMUIR, int MODE, int FLOW, bool WS = false, bool EDGE = true>
 __device__ __forceinline__ bool step_tile(const Phys& p, const TileIO& io, unsigned char* sm, float2* PP,
-                                          unsigned long long* mbar, uint32_t parity, int x0, int y0) {
+                                          unsigned long long* mbar, uint32_t parity, int x0, int y0, int t, int bar,
+                                          bool late) {
     using T = Traits<ST>;
     using S = Smem<ST>;
     using P = typename T::P;
@@ -789,9 +811,8 @@ __device__ __forceinline__ bool step_tile(const Phys& p, const TileIO& io, unsig
     static_assert(CPT == 1 || T::kPair16, "two cells per thread only for 16-bit pairs");
     const P* FG = reinterpret_cast<const P*>(sm + S::FG);
     const float2* Hist = reinterpret_cast<const float2*>(sm + S::HIST);
-    const int t = threadIdx.x;
     if constexpr (!WS) __syncthreads();
-    bool abort = !mbar_wait_bounded(mbar, parity);
+    bool abort = WS ? late : !mbar_wait_bounded(mbar, parity);
 
     const int tx = (t % G::TPR) * CPT, ty = t / G::TPR;
     const int x = x0 + tx, y = y0 + ty;
@@ -799,20 +820,21 @@ __device__ __forceinline__ bool step_tile(const Phys& p, const TileIO& io, unsig
     const bool act1 = CPT == 2 && (!EDGE || (active && x + 1 < p.nx));  // the thread's second cell
     const long long cell = p.org + (long long)y * p.pitch + x;
     // mass flux of the previous step (density ratio != 1 only; the own cells', read early so that
-    // its latency overlaps the stencil work)
+    // its latency overlaps the stencil work; past L1, since a launch of several steps reads what
+    // another SM wrote during the launch)
     C Spx = bcv<C>(0.f), Spy = bcv<C>(0.f);
     if constexpr (var) {
         if (!io.first && active) {
             if constexpr (CPT == 1) {
-                const float2 s = io.shist_src[cell];
+                const float2 s = __ldcg(io.shist_src + cell);
                 Spx = s.x;
                 Spy = s.y;
             } else if (act1) {
-                const float4 s = *reinterpret_cast<const float4*>(io.shist_src + cell);
+                const float4 s = __ldcg(reinterpret_cast<const float4*>(io.shist_src + cell));
                 Spx = make_float2(s.x, s.z);
                 Spy = make_float2(s.y, s.w);
             } else {
-                const float2 s = io.shist_src[cell];
+                const float2 s = __ldcg(io.shist_src + cell);
                 Spx = make_float2(s.x, 0.f);
                 Spy = make_float2(s.y, 0.f);
             }
@@ -855,13 +877,13 @@ __device__ __forceinline__ bool step_tile(const Phys& p, const TileIO& io, unsig
         for (int i = 0; i < 9; ++i) r[i] = base[i * SLOT - cx(i)];
         PP[ey * G::EXP + ex + G::PPO] = pair_sum1<ST>(r, make_float2(T::kPair16 ? p.phi_ref : 0.f, 0.f));
     }
-    if (WS ? compute_sync_or<G::NT>(abort) : __syncthreads_or(abort)) {
+    if (WS ? compute_sync_or<G::NT>(bar, abort) : __syncthreads_or(abort)) {
         // a staging copy did not arrive in time: report it, wait (bounded) for it, store nothing
         if (t == 0) {
             atomicOr(io.status, kStatusTimeout);
             mbar_wait_bounded(mbar, parity);
         }
-        if constexpr (WS) compute_sync<G::NT>();
+        if constexpr (WS) compute_sync<G::NT>(bar);
         else __syncthreads();
         return true;
     }
@@ -1402,10 +1424,11 @@ template <int ST> __device__ __forceinline__ bool tile_is_interior(const Phys& p
 // step_tile on the interior or the edge path (the choice is uniform over the tile).
 template <int ST, bool WALLS, bool LANGMUIR, int MODE, int FLOW, bool WS = false>
 __device__ __forceinline__ bool step_tile_any(const Phys& p, const TileIO& io, unsigned char* sm, float2* PP,
-                                              unsigned long long* mbar, uint32_t parity, int x0, int y0) {
+                                              unsigned long long* mbar, uint32_t parity, int x0, int y0, int t,
+                                              int bar = 0, bool late = false) {
     if (tile_is_interior<ST>(p, x0, y0))
-        return step_tile<ST, WALLS, LANGMUIR, MODE, FLOW, WS, false>(p, io, sm, PP, mbar, parity, x0, y0);
-    return step_tile<ST, WALLS, LANGMUIR, MODE, FLOW, WS, true>(p, io, sm, PP, mbar, parity, x0, y0);
+        return step_tile<ST, WALLS, LANGMUIR, MODE, FLOW, WS, false>(p, io, sm, PP, mbar, parity, x0, y0, t, bar, late);
+    return step_tile<ST, WALLS, LANGMUIR, MODE, FLOW, WS, true>(p, io, sm, PP, mbar, parity, x0, y0, t, bar, late);
 }
 
 // Resident CTAs per SM that the one-tile kernels (step_kernel, and batch_step_kernel but for the
@@ -1444,7 +1467,7 @@ __global__ void __launch_bounds__(GeoOf<ST>::NT, tile_min_blocks<ST>(FLOW)) step
     cudaGridDependencySynchronize();
     if (threadIdx.x == 0) issue_tile_loads<ST, FLOW>(sm, &a.tm_fg, &a.tm_h, &a.tm_hist, x0, y0, mbar);
     step_tile_any<ST, WALLS, LANGMUIR, MODE, FLOW>(a.p, a.io, sm, reinterpret_cast<float2*>(sm + Smem<ST>::PP), mbar, 0,
-                                                   x0, y0);
+                                                   x0, y0, (int)threadIdx.x);
 }
 
 // Tile k of a grid of ntx x nty tiles: rows in the order first, last, then the interior (the two
@@ -1538,7 +1561,7 @@ __device__ __forceinline__ void step_pipe_body(const StepArgs& a, int ntx, int n
         const int b = it & 1;
         const uint32_t parity = (uint32_t)(it >> 1) & 1u;
         const bool late = !mbar_wait_bounded(&full[b], parity);
-        if (compute_sync_or<G::NT>(late)) {  // uniform: a copy (or the stop mark) did not come in time
+        if (compute_sync_or<G::NT>(1, late)) {  // uniform: a copy (or the stop mark) did not come in time
             if (threadIdx.x == 0) {
                 atomicOr(a.io.status, kStatusTimeout);
                 // wait (bounded) for the copies that may still be in flight into either buffer
@@ -1551,7 +1574,7 @@ __device__ __forceinline__ void step_pipe_body(const StepArgs& a, int ntx, int n
         if (x0 < 0) break;  // uniform: every compute thread reads the same slot
         float2* PP = reinterpret_cast<float2*>(sm + S::PIPE_PP + b * S::PP_BYTES);
         if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(a.p, a.io, sm + b * S::STAGE, PP, &full[b], parity, x0,
-                                                                  y0))
+                                                                  y0, (int)threadIdx.x, 1))
             break;  // uniform (decided by the OR barrier inside)
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[b]);  // this warp is done with buffer b
@@ -1569,6 +1592,404 @@ __global__ void __maxnreg__(pipe_regs2(FLOW)) step_kernel_pipe2(const __grid_con
 template <int ST, bool WALLS, bool LANGMUIR, int FLOW> constexpr auto pipe_kernel() {
     if constexpr (cpt_of(ST) == 1) return step_kernel_pipe<ST, WALLS, LANGMUIR, FLOW>;
     else return step_kernel_pipe2<ST, WALLS, LANGMUIR, FLOW>;
+}
+
+// ---- a run of steps of one lattice in one launch ----
+struct RunArgs {
+    CUtensorMap tm_fg[2], tm_h[2], tm_hist[2];  // of each buffer
+    Phys p;
+    void* pops[2];
+    float2* hist[2];
+    float2* shist[2];
+    unsigned* status;
+    long long steps;          // steps taken before this launch
+    int cur, first;           // buffer of the current state; 1 on the first step after initialisation
+    int nsteps;               // steps of this launch
+    int ntx, nty;             // tiles
+    int depth, lag;           // levels of a pass and the tile rows between successive levels (see RunWalk)
+    int reach;                // tile rows above and below a tile that its step reads
+    int ring;                 // tile buffers used, 1 .. RunShape::NB
+    int ahead;                // tile j waits in the lead warp until tile j - ahead is signalled (>= ring)
+    int batch;                // tiles per round of the lead warp, 1 .. 8 (4 with a reach of two)
+    unsigned* ctr;            // tile counter of this launch (zero at start), or null: fixed positions
+    unsigned* rows;           // tiles finished per tile row (zero at start)
+};
+
+// Shape of the persistent CTA: NG compute groups of NT threads, each updating its own tile, NB tile
+// buffers that TMA fills ahead of them, and four more warps (lead, signal and two copy warps).
+template <int ST, int FLOW> struct RunShape {
+    using G = GeoOf<ST>;
+    using S = Smem<ST>;
+    static constexpr int WPG = G::NT / 32;
+    static constexpr int NG = cpt_of(ST) == 1 ? (FLOW == kFlowVarRho ? 2 : 3) : (FLOW == kFlowVarRho ? 3 : 4);
+    static constexpr int THREADS = NG * G::NT + 128;
+    static constexpr int STAGE = FLOW ? S::PP : S::H;
+    static constexpr int PP_ALL = 2 * NG * S::PP_BYTES;  // two (phi, psi) tiles per group, used in turn
+    static constexpr int MAX_SMEM = 227 * 1024;
+    static constexpr int NB_FIT = (MAX_SMEM - PP_ALL - 44 * 8 * NG) / STAGE;
+    static constexpr int NB = NB_FIT < 8 ? NB_FIT : 8;
+    static constexpr int DB = 8;                     // queue entries per group, used in turn
+    static constexpr int QN = NG * DB;
+    static constexpr int PP = NB * STAGE;
+    static constexpr int QUEUE = PP + PP_ALL;        // int4 per entry: x0 (-1: stop), y0, source buffer | first << 1, seed
+    static constexpr int BAR = QUEUE + 16 * QN;      // queued, full and done barrier of each entry
+    static constexpr int SIG = BAR + 24 * QN;        // int per entry: how often it was signalled
+    static constexpr int BYTES = SIG + 4 * QN;
+    static_assert(NB >= NG && NB <= DB, "a buffer per group; queue entries for every buffer in use");
+    static_assert(BYTES <= MAX_SMEM, "shared memory of one CTA");
+};
+
+// The order of the tiles of a launch of several steps.  Level s is step s of the launch; a tile of
+// level s reads what level s - 1 wrote in its own and its neighbouring tile rows, and overwrites what
+// level s - 1 read there.  The levels are cut into passes of `depth`; within a pass, wave w holds tile
+// row index w - s lag of every level s of the pass, so that a row is updated `depth` times while it
+// is in L2 (depth 1: one level after the other).  Row index i of level s is tile row i between
+// walls and, with a periodic y, row i + s reach around the ring: then every row that a tile
+// depends on, also across the periodic edge, comes before it in this order.
+struct RunWalk {
+    int base, levels;         // first level and levels of the pass
+    int w, before;            // wave, and rows in the waves of the pass before it
+    int lo, lo_left;          // first level with a row in wave w, and the waves until it ends
+    int hi, hi_left;          // last level with a row in wave w, and the waves until the next begins
+    int turn;                 // periodic y: base reach mod nty
+    int q, col;               // row number in the pass, tile column
+    int level, row;           // level and tile row of the current position (level >= nsteps: past the end)
+    __device__ __forceinline__ void enter(const RunArgs& a) {
+        levels = min(a.depth, a.nsteps - base);
+        w = before = lo = hi = 0;
+        lo_left = a.nty;
+        hi_left = a.lag;
+    }
+    // start at position k, then move on by dq rows and dc columns (dc < ntx)
+    template <bool WALLS> __device__ __forceinline__ void start(const RunArgs& a, int k) {
+        base = turn = 0;
+        enter(a);
+        q = k / a.ntx;
+        col = k - q * a.ntx;
+        settle<WALLS>(a);
+    }
+    template <bool WALLS> __device__ __forceinline__ void move(const RunArgs& a, int dq, int dc) {
+        q += dq;
+        col += dc;
+        if (col >= a.ntx) {
+            col -= a.ntx;
+            ++q;
+        }
+        settle<WALLS>(a);
+    }
+    template <bool WALLS> __device__ __forceinline__ void settle(const RunArgs& a) {
+        while (q >= levels * a.nty && base < a.nsteps) {
+            q -= levels * a.nty;
+            base += levels;
+            if (!WALLS) turn = (int)((turn + (long long)levels * a.reach) % a.nty);
+            enter(a);
+        }
+        int s = 0, i = q;
+        if (levels > 1) {
+            for (; q >= before + hi - lo + 1;) {
+                before += hi - lo + 1;
+                ++w;
+                if (--lo_left == 0) {
+                    ++lo;
+                    lo_left = a.lag;
+                }
+                if (--hi_left == 0) {
+                    hi_left = a.lag;
+                    if (hi < levels - 1) ++hi;
+                }
+            }
+            s = lo + q - before;
+            i = w - s * a.lag;
+        }
+        level = base + s;
+        row = i;
+        if (!WALLS)
+            for (row += turn + s * a.reach; row >= a.nty;) row -= a.nty;
+    }
+};
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int ld_shared_acquire(const int* p) {
+    int v;
+    asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];\n" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_shared_release(int* p, int v) {
+    asm volatile("st.release.cta.shared::cta.s32 [%0], %1;\n" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+constexpr unsigned kRowPollLimit = 1u << 23;  // polls of 0.1 us or more: the wait ends within seconds
+
+// A run of steps by a persistent, warp-specialised grid of one CTA per SM.  Between steps the grid's
+// tiles wait for their neighbours only, through counters in global memory: no launch, no drained
+// grid and no empty last wave between steps, and with depth > 1 a row is updated several times
+// while it is in L2.  Sheared drop, us per step, one launch per step / a run: FP32 128 x 128 4.3 / 4.0,
+// 512 x 256 6.6 / 5.5, 608 x 512 10.4 / 8.3, 2048 x 1024 73.2 / 67.1 (one level at a time 68.8, which
+// is the measured copy rate); FP16 1024 x 512 14.7 / 12.4, 2048 x 1024 50.3 / 43.3; BF16_FG
+// 1531 x 787 35.6 / 28.4.  One group of CTAs per tile and step left the SM idle between a tile's
+// copy and its arithmetic; here three groups (FP32; four of half the threads with two cells per
+// thread) have their next tiles in shared memory.
+// What bounds it: FP32 storage HBM and L2 latency (five buffers of 41 KB fill the SM), 16-bit storage
+// the support warps and the issue rate about equally (0.8 us per tile and SM).
+// Roles of the CTA's warps.  A CTA takes positions of RunWalk's order, claimed from a counter or (small
+// grids) c, c + CTAs, .. for CTA c, as its tiles j = 0, 1, ..
+//   Lead warp: finds the tiles, waits until the rows that each reads are complete, and queues them.
+//   Copy warps (two, one lane each): stage a queued tile's boxes with TMA, half each, into buffer
+//     j mod ring once tile j - ring is done, on the tile's "full" barrier.  A box takes a lane 40 ns,
+//     whatever its size, and a tile's waits 0.5 us: with one lane the FP16 step took 57 us.
+//   Compute groups: group g updates the tiles j = g, g + ng, .. and arrives on their "done" barrier
+//     (one arrival per warp).  The copies and the barrier of one group's tile overlap the arithmetic
+//     of the others.
+//   Signal warp (one lane per group): adds one to the tile row's counter for every tile done, with
+//     release order: its stores become visible first, which takes 1 to 2 us under load, so no other
+//     warp waits for that (with a fence per tile in the lead warp the step took twice as long).
+// Tile j = m ng + g uses entry m mod DB of group g: its place in the queue and its three barriers.  The
+// lead fills it again only when the entry's last tile has been signalled, so by then nobody waits
+// for an earlier phase of its barriers, and each waiting warp follows every phase of a barrier in
+// turn (a parity tells two successive phases apart, no more).
+// No tile waits for one later in the order, and a CTA stages and updates its tiles in that order, so
+// the earliest tile can always run: with claimed positions whichever CTAs are resident, with fixed ones
+// while all are (such launches are cooperative).  Every wait is bounded; a copy lane that gives up
+// waits (bounded) for its copies.
+template <int ST, bool WALLS, bool LANGMUIR, int FLOW>
+__global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
+    step_kernel_run(const __grid_constant__ RunArgs a) {
+    using Sh = RunShape<ST, FLOW>;
+    using S = Smem<ST>;
+    using G = GeoOf<ST>;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(sm + Sh::BAR);
+    unsigned long long* done = full + Sh::QN;
+    unsigned long long* queued = done + Sh::QN;
+    int* signalled = reinterpret_cast<int*>(sm + Sh::SIG);
+    int4* queue = reinterpret_cast<int4*>(sm + Sh::QUEUE);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < Sh::QN; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&done[i], Sh::WPG);
+            mbar_init(&queued[i], 1);
+            signalled[i] = 0;
+            queue[i] = make_int4(0, 0, 0, 0);
+        }
+        fence_mbar_init();
+    }
+    __syncthreads();
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();
+    const int ring = a.ring, ng = min(Sh::NG, ring);
+    const int warp = (int)threadIdx.x / 32, lane = (int)threadIdx.x % 32;
+    // an index that runs around a ring, and the parity of its turn
+    auto advance = [](int& i, uint32_t& parity, int n, int size) {
+        for (i += n; i >= size; i -= size) parity ^= 1u;
+    };
+    // entries of successive tiles of the CTA, and the parity of their barriers' phases
+    struct Seq {
+        int g = 0, d = 0;
+        uint32_t parity = 0u;
+        __device__ __forceinline__ int index() const { return g * Sh::DB + d; }
+        __device__ __forceinline__ void next(int ng) {
+            if (++g == ng) {
+                g = 0;
+                if (++d == Sh::DB) {
+                    d = 0;
+                    parity ^= 1u;
+                }
+            }
+        }
+    };
+
+    if (warp == Sh::NG * Sh::WPG) {
+        // ---- lead warp: `batch` tiles at a time.  `share` successive lanes hold one of them, four for a
+        // reach of one and eight for two; each asks for the counter of one of the tile rows around
+        // it, so one round trip tells of all. ----
+        const int total = a.nsteps * a.ntx * a.nty;
+        const int share = a.reach > 1 ? 8 : 4;
+        const int off = lane % share - a.reach, n_own = lane / share;
+        const unsigned mine = (1u << share) - 1u;
+        const int step = a.ctr ? 1 : (int)gridDim.x;
+        const unsigned by_ng = ng > 1 ? 0xFFFFFFFFu / (unsigned)ng + 1u : 0u;  // j / ng as a product
+        auto turn_of = [&](int j, int& e) {  // entry of tile j, and how often it was filled before
+            const int m = ng > 1 ? (int)__umulhi((unsigned)j, by_ng) : j;
+            e = (j - m * ng) * Sh::DB + m % Sh::DB;
+            return m / Sh::DB;
+        };
+        auto claim = [&]() { return lane == 0 ? (int)atomicAdd(a.ctr, (unsigned)a.batch) : 0; };
+        int pos = a.ctr ? __shfl_sync(0xffffffffu, claim(), 0) : (int)blockIdx.x;
+        RunWalk walk;
+        walk.start<WALLS>(a, pos + n_own * step);
+        const int dq = a.batch * step / a.ntx, dc = a.batch * step - dq * a.ntx;  // of a round with fixed positions
+        for (int j0 = 0, left = 1; left; j0 += a.batch) {
+            const int later = a.ctr ? claim() : 0;  // the next claim, early (lane 0)
+            const bool live = pos + n_own * step < total && n_own < a.batch;
+            const unsigned count = __popc(__ballot_sync(0xffffffffu, live)) / share;
+            left = count == a.batch;  // else the order ends in this round: stop marks follow, one per group
+            // the first lane of a tile queues it; the one past the last tile queues the stop marks
+            const int own = live ? 1 : (left || n_own != (int)count ? 0 : ng);
+            const int j = j0 + n_own;
+            int4 entry = make_int4(-1, 0, 0, 0);
+            bool open = true;  // this lane's row is complete
+            const unsigned* rows = a.rows;
+            const unsigned need = (unsigned)walk.level * (unsigned)a.ntx;
+            if (live) {
+                entry = make_int4(walk.col * G::TX, walk.row * G::TY, ((a.cur + walk.level) & 1) | (walk.level == 0 && a.first ? 2 : 0),
+                                  Traits<ST>::kPair16 ? (int)step_seed(a.steps + walk.level) : 0);
+                open = walk.level == 0 || off > a.reach;
+                int r = walk.row + off;
+                if (WALLS) r = min(max(r, 0), a.nty - 1);
+                else if (r < 0 || r >= a.nty) r = (r + 2 * a.nty) % a.nty;
+                rows += r;
+            }
+            // queue each tile as soon as its rows and a queue entry are ready
+            int put = lane % share == 0 ? 0 : own;
+            for (unsigned it = 0; __any_sync(0xffffffffu, put < own); ++it) {
+                if (it > 64) __nanosleep(100);
+                if (!open) open = ld_acquire(rows) >= need;
+                const unsigned ready = __ballot_sync(0xffffffffu, open);
+                __syncwarp();
+                if (put < own && (ready >> lane & mine) == mine) {
+                    int e, k;
+                    const int turn = turn_of(j + put, e), last = turn_of(max(j + put - a.ahead, 0), k);
+                    if ((turn == 0 || ld_shared_acquire(&signalled[e]) >= turn) &&
+                        (j + put < a.ahead || ld_shared_acquire(&signalled[k]) > last)) {
+                        queue[e] = entry;
+                        mbar_arrive(&queued[e]);
+                        ++put;
+                    }
+                }
+                if (it == kRowPollLimit) {
+                    if (lane == 0) atomicOr(a.status, kStatusTimeout);
+                    return;
+                }
+            }
+            if (!left) return;
+            if (a.ctr) {
+                const int was = pos;
+                pos = __shfl_sync(0xffffffffu, later, 0);
+                const int q = (pos - was) / a.ntx;
+                walk.move<WALLS>(a, q, pos - was - q * a.ntx);
+            } else {
+                pos += a.batch * step;
+                walk.move<WALLS>(a, dq, dc);
+            }
+        }
+        return;
+    }
+    if (warp > Sh::NG * Sh::WPG + 1) {
+        // ---- copy warps ----
+        if (lane != 0) return;
+        const bool first = warp == Sh::NG * Sh::WPG + 2;
+        Seq tile, last;  // the tile at hand, and the one `ring` before it
+        int b = 0, stops = 0;
+        uint32_t unused = 0u;
+        for (int j = 0;; ++j, tile.next(ng), advance(b, unused, 1, ring)) {
+            bool ok = mbar_wait_bounded(&queued[tile.index()], tile.parity);
+            const int4 e = queue[tile.index()];
+            if (ok && e.x < 0) {
+                if (!first) return;
+                mbar_arrive(&full[tile.index()]);  // no copy: the group reads the stop mark
+                if (++stops == ng) return;
+                continue;
+            }
+            if (ok && j >= ring) {
+                ok = mbar_wait_bounded(&done[last.index()], last.parity);
+                if (ok) last.next(ng);
+            }
+            if (!ok) {
+                atomicOr(a.status, kStatusTimeout);
+                for (; last.index() != tile.index(); last.next(ng)) mbar_wait_bounded(&full[last.index()], last.parity);
+                return;
+            }
+            // the stores that the row counters tell of (generic proxy) before these copies (async proxy)
+            asm volatile("fence.proxy.async.global;\n" ::: "memory");
+            const int src = e.z & 1;
+            unsigned char* stage = sm + b * Sh::STAGE;
+            if (first) {
+                // (the other half may have begun to arrive: the barrier waits for this arrival)
+                mbar_expect_tx(&full[tile.index()], FLOW ? S::TX_BYTES : S::TX_BYTES_NOH);
+                issue_boxes<ST, FLOW, 0, 2>(stage, &a.tm_fg[src], &a.tm_h[src], &a.tm_hist[src], e.x, e.y, &full[tile.index()]);
+            } else {
+                issue_boxes<ST, FLOW, 1, 2>(stage, &a.tm_fg[src], &a.tm_h[src], &a.tm_hist[src], e.x, e.y, &full[tile.index()]);
+            }
+        }
+    }
+    if (warp == Sh::NG * Sh::WPG + 1) {
+        // ---- signal warp: lane g follows group g ----
+        const int own = (lane < ng ? lane : 0) * Sh::DB;
+        int d = 0, turns = 0;
+        bool live = lane < ng;
+        uint32_t parity = 0u;
+        for (unsigned idle = 0; __any_sync(0xffffffffu, live);) {
+            int row = -1;
+            const bool moved = live && mbar_test(&done[own + d], parity);
+            if (moved) {
+                const int4 e = queue[own + d];
+                live = e.x >= 0;
+                row = live ? e.y / G::TY : -1;
+            }
+            if (__any_sync(0xffffffffu, moved)) {
+                idle = 0;
+                // the tile's stores, which the group's arrivals tell of, before the count
+                if (row >= 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(a.rows + row) : "memory");
+                if (moved) {
+                    st_shared_release(&signalled[own + d], turns + 1);
+                    if (++d == Sh::DB) {
+                        d = 0;
+                        parity ^= 1u;
+                        ++turns;
+                    }
+                }
+            } else {
+                if (++idle == kRowPollLimit) {
+                    if (lane == 0) atomicOr(a.status, kStatusTimeout);
+                    return;
+                }
+                __nanosleep(40);
+            }
+        }
+        return;
+    }
+
+    // ---- compute groups ----
+    const int g = (int)threadIdx.x / G::NT, t = (int)threadIdx.x - g * G::NT;
+    if (g >= ng) return;
+    int b = g;
+    for (unsigned m = 0;; ++m) {
+        const int at = g * Sh::DB + (int)(m % Sh::DB);
+        unsigned long long* mbar = &full[at];
+        const uint32_t parity = m / Sh::DB & 1u;
+        const bool late = !mbar_wait_bounded(mbar, parity);
+        __syncwarp();
+        const int4 e = queue[at];
+        if (e.x < 0) {
+            // the stop mark; the barrier meets the one in step_tile, should another thread's wait have
+            // given up before it saw the mark
+            if (compute_sync_or<G::NT>(1 + g, late)) compute_sync<G::NT>(1 + g);
+            else if (lane == 0) mbar_arrive(&done[at]);
+            return;
+        }
+        const int src = e.z & 1;
+        TileIO io;
+        io.src = nullptr;
+        io.hist_src = nullptr;
+        io.dst = src ? a.pops[0] : a.pops[1];
+        io.hist_dst = src ? a.hist[0] : a.hist[1];
+        io.shist_src = src ? a.shist[1] : a.shist[0];
+        io.shist_dst = src ? a.shist[0] : a.shist[1];
+        io.status = a.status;
+        io.out[0] = io.out[1] = io.out[2] = io.out[3] = io.out[4] = nullptr;
+        io.seed = (unsigned)e.w;
+        io.first = e.z >> 1;
+        float2* PP = reinterpret_cast<float2*>(sm + Sh::PP + (2 * g + (int)(m & 1u)) * S::PP_BYTES);
+        if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(a.p, io, sm + b * Sh::STAGE, PP, mbar, parity, e.x, e.y, t,
+                                                                  1 + g, late))
+            return;  // uniform (decided by the OR barrier inside)
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&done[at]);
+        for (b += ng; b >= ring;) b -= ring;
+    }
 }
 
 // ---- many lattices in one launch ----
@@ -1641,7 +2062,8 @@ __global__ void __launch_bounds__(GeoOf<ST>::NT, batch_min_blocks<ST>(FLOW)) bat
     io.out[0] = io.out[1] = io.out[2] = io.out[3] = io.out[4] = nullptr;
     io.seed = step_seed(d.steps + b.s);
     io.first = d.first && b.s == 0;
-    step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW>(*sp, io, sm, reinterpret_cast<float2*>(sm + S::PP), mbar, 0, x0, y0);
+    step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW>(*sp, io, sm, reinterpret_cast<float2*>(sm + S::PP), mbar, 0, x0, y0,
+                                                    (int)threadIdx.x);
 }
 
 // One step of many lattices by a persistent, warp-specialised grid (the design of step_kernel_pipe).
@@ -1729,7 +2151,7 @@ __device__ __forceinline__ void batch_ws_body(const BatchArgs& b) {
         const int q = it & 1;
         const uint32_t parity = (uint32_t)(it >> 1) & 1u;
         const bool late = !mbar_wait_bounded(&full[q], parity);
-        if (compute_sync_or<G::NT>(late)) {
+        if (compute_sync_or<G::NT>(1, late)) {
             if (threadIdx.x == 0) {
                 flag_batch_timeout(b);
                 mbar_wait_bounded(&full[q], parity);
@@ -1754,7 +2176,8 @@ __device__ __forceinline__ void batch_ws_body(const BatchArgs& b) {
         io.first = d.first && b.s == 0;
         const Phys& p = *reinterpret_cast<const Phys*>(sm + S::BWS_PHYS + q * S::PHYS_BYTES);
         float2* PP = reinterpret_cast<float2*>(sm + S::PIPE_PP + q * S::PP_BYTES);
-        if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(p, io, sm + q * S::STAGE, PP, &full[q], parity, x0, y0))
+        if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(p, io, sm + q * S::STAGE, PP, &full[q], parity, x0, y0,
+                                                                  (int)threadIdx.x, 1))
             return;
         __syncwarp();
         if ((threadIdx.x & 31) == 0) mbar_arrive(&empty[q]);

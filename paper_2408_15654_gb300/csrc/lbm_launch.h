@@ -21,6 +21,11 @@ inline TileDims tile_dims(int st) {
     return TileDims{Geo<2>::TX, Geo<2>::TY, Geo<2>::BW, Geo<2>::BH, Geo<2>::TX + 2 * hx0};
 }
 
+// Of step_kernel_run: resident CTAs per SM, and tile buffers per CTA.
+struct RunDims {
+    int blocks_per_sm, buffers;
+};
+
 // Runtime flags of a launch, mapped to the kernel variant.
 struct Variant {
     bool walls, langmuir, flow, var_rho;
@@ -88,6 +93,33 @@ cudaError_t launch_step_impl(const StepArgs& a, int mode, const Variant& v, dim3
     return dispatch_variant(v, [&]<bool W, bool L, int F>() {
         if (mode == kStep) return cudaLaunchKernelEx(&cfg, step_kernel<ST, W, L, kStep, F>, a);
         return cudaLaunchKernelEx(&cfg, step_kernel<ST, W, L, kMoments, F>, a);
+    });
+}
+
+// A run of steps on `ctas` CTAs, at most one per SM.  With fixed positions (no tile counter) every CTA
+// needs every other, so the launch is cooperative; it follows the counters' reset, so there is no
+// launch before it to overlap with.
+template <int ST>
+cudaError_t launch_run_impl(const RunArgs& a, const Variant& v, int ctas, cudaStream_t stream) {
+    cudaLaunchAttribute attr[1];
+    return dispatch_variant(v, [&]<bool W, bool L, int F>() {
+        using Sh = RunShape<ST, F>;
+        cudaLaunchConfig_t cfg = pdl_config(dim3((unsigned)ctas), Sh::BYTES, stream, attr, Sh::THREADS);
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = a.ctr ? 0 : 1;
+        return cudaLaunchKernelEx(&cfg, step_kernel_run<ST, W, L, F>, a);
+    });
+}
+
+// Opt the run kernel of variant v into its shared memory and describe it.
+template <int ST> cudaError_t prepare_run_impl(const Variant& v, RunDims* d) {
+    return dispatch_variant(v, [&]<bool W, bool L, int F>() {
+        using Sh = RunShape<ST, F>;
+        d->buffers = Sh::NB;
+        auto k = step_kernel_run<ST, W, L, F>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::BYTES);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->blocks_per_sm, k, Sh::THREADS, Sh::BYTES);
+        return e;
     });
 }
 
@@ -168,6 +200,8 @@ cudaError_t prepare_batch_impl(int* ws_blocks_per_sm) {
 // Entry points of the per-storage translation units; st is the storage mode.
 cudaError_t launch_step(int st, const StepArgs& a, int mode, const Variant& v, dim3 grid, int pipe, cudaStream_t s);
 cudaError_t prepare_step(int st, const Variant& v, int* blocks_per_sm, int* pipe_blocks_per_sm);
+cudaError_t launch_run(int st, const RunArgs& a, const Variant& v, int ctas, cudaStream_t s);
+cudaError_t prepare_run(int st, const Variant& v, RunDims* d);
 cudaError_t launch_batch(int st, const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s);
 cudaError_t prepare_batch(int st, int* ws_blocks_per_sm);
 
@@ -175,6 +209,8 @@ cudaError_t prepare_batch(int st, int* ws_blocks_per_sm);
     cudaError_t launch_step_##name(const StepArgs& a, int mode, const Variant& v, dim3 grid, int pipe,              \
                                    cudaStream_t s);                                                                \
     cudaError_t prepare_step_##name(const Variant& v, int* blocks_per_sm, int* pipe_blocks_per_sm);                 \
+    cudaError_t launch_run_##name(const RunArgs& a, const Variant& v, int ctas, cudaStream_t s);                    \
+    cudaError_t prepare_run_##name(const Variant& v, RunDims* d);                                                   \
     cudaError_t launch_batch_##name(const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s);         \
     cudaError_t prepare_batch_##name(int* ws_blocks_per_sm);
 LBM_DECLARE_STORAGE(fp32)
@@ -193,6 +229,10 @@ LBM_DECLARE_STORAGE(bf16fg)
     cudaError_t prepare_step_##name(const Variant& v, int* blocks_per_sm, int* pipe_blocks_per_sm) {                \
         return prepare_step_impl<ST>(v, blocks_per_sm, pipe_blocks_per_sm);                                       \
     }                                                                                                              \
+    cudaError_t launch_run_##name(const RunArgs& a, const Variant& v, int ctas, cudaStream_t s) {                   \
+        return launch_run_impl<ST>(a, v, ctas, s);                                                                 \
+    }                                                                                                              \
+    cudaError_t prepare_run_##name(const Variant& v, RunDims* d) { return prepare_run_impl<ST>(v, d); }             \
     cudaError_t launch_batch_##name(const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s) {        \
         return launch_batch_impl<ST>(b, v, ntiles, s);                                                            \
     }                                                                                                              \
