@@ -255,11 +255,11 @@ int lbm_get_kernel(const lbm_handle* h, int* variant);
  * valid until the next call on the same thread. */
 const char* lbm_last_error(void);
 
-/* ---- many lattices in one launch per step --------------------------------------------------
+/* ---- many lattices in one launch -----------------------------------------------------------
  * Not in the paper, which treats one lattice at a time: a batch advances many independent
- * lattices (lbm_handle members, each with its own parameters, grid and workspace) by one launch
- * of one kernel per step and per group of members that share storage mode, boundary kind and
- * EOS.  Every member's result is bit for bit the one lbm_step gives it alone: a cell's update
+ * lattices (lbm_handle members, each with its own parameters, grid and workspace), by group of
+ * members that share storage mode, boundary kind and EOS: a run of many steps of a group in one
+ * launch, or one launch per step and group (see lbm_batch_set_kernel).  Every member's result is bit for bit the one lbm_step gives it alone: a cell's update
  * depends only on its lattice's buffers, constants and step count, never on the schedule.
  * Ownership: the caller owns the batch workspace and the members; members stay valid and are
  * not destroyed while they belong to a batch (lbm_batch_set_members replaces the list).  All
@@ -293,7 +293,7 @@ int lbm_batch_create(int max_members, int64_t max_tiles, void* d_workspace, size
 int lbm_batch_set_members(lbm_batch* b, lbm_handle* const* members, int n);
 
 /* Order of the tiles (LBM_SCHED_*) and the number of steps per captured CUDA graph (0: plain
- * launches).  Default: LBM_SCHED_LARGEST_FIRST, no graph. */
+ * launches) where a step is a launch per group (see lbm_batch_set_kernel).  Default: LBM_SCHED_LARGEST_FIRST, no graph. */
 int lbm_batch_set_schedule(lbm_batch* b, int schedule, int graph_steps);
 
 /* Advance every member by n steps (asynchronous, like lbm_step).  Each member's device status
@@ -301,7 +301,7 @@ int lbm_batch_set_schedule(lbm_batch* b, int schedule, int graph_steps);
 int lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Time each schedule with 16-step graphs, and the fastest of them without a graph, over about
- * trial_steps steps each, and keep the fastest.  The trials are real steps: every member
+ * trial_steps steps each, one launch per step and group, and keep the fastest.  The trials are real steps: every member
  * advances by 4 * (16 + trial_steps rounded up to a multiple of 16) + 1 + trial_steps steps
  * (without graphs, on the legacy default stream: 4 * (1 + trial_steps)).  Synchronous. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_steps);
@@ -311,8 +311,10 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_
  *   LBM_KERNEL_PIPELINED  persistent, warp-specialised CTAs: a copy warp claims tiles from a
  *                         counter in the workspace and stages each tile's boxes and its lattice's
  *                         constants while the compute warps work on the previous tile;
- *   LBM_KERNEL_AUTO       the default: PIPELINED for every group (the faster one on GB300
- *                         with a 64-lattice mix in every storage mode).
+ *   LBM_KERNEL_AUTO       the default: PIPELINED for calls of fewer than eight steps; from eight
+ *                         steps on, runs of many steps in one launch, members of ten tiles per SM or
+ *                         more one by one as lbm_step does them, the others together.  Batches of
+ *                         16-bit lattices with one to three tiles per SM in all keep PIPELINED.
  * PIPELINED applies only if it fits (else TILE).  lbm_batch_get_kernel reports the setting. */
 int lbm_batch_set_kernel(lbm_batch* b, int variant);
 int lbm_batch_get_kernel(const lbm_batch* b, int* variant);

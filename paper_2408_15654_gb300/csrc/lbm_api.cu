@@ -289,14 +289,9 @@ int launch_step(lbm_handle* h, int mode, double* const out[5]) {
     cudaError_t e = lbm::launch_step(h->prm.storage, a, mode, variant_of(h->prm, h->phys.var_rho != 0), grid, pipe,
                                      h->stream);
     if (e != cudaSuccess) return fail(LBM_ECUDA, "step launch: %s", cudaGetErrorString(e));
+    if (mode == lbm::kStep) h->launches++;
     return LBM_OK;
 }
-
-// Counters of a run of steps: the tile counter, then the row counters.  They share the reduction's
-// partial sums (work of one handle is ordered on its stream).
-constexpr int kRowOffset = 32, kRowCounters = 2016;
-static_assert((kRowOffset + kRowCounters) * sizeof(unsigned) <= lbm::kMaxPartials * sizeof(double),
-              "the counters fit the partial sums");
 
 // Whether `n` steps in a row go as runs (one launch for many steps).  Always the faster way but for a
 // few steps, whose launch and counters' reset cost more than they save (at 128 x 128: 4.3 us per step
@@ -377,6 +372,7 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     h->last_pipe_step = -2;
     cudaError_t e = lbm::launch_run(h->prm.storage, a, variant_of(h->prm, h->phys.var_rho != 0), ctas, h->stream);
     if (e != cudaSuccess) return fail(LBM_ECUDA, "run launch: %s", cudaGetErrorString(e));
+    h->launches++;
     return LBM_OK;
 }
 

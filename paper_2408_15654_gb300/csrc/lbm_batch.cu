@@ -1,8 +1,9 @@
-// Many independent lattices advanced together: one launch of the many-lattice kernel per step
-// and per group of lattices that share a storage mode, boundary kind and EOS.  The workspace
-// holds a descriptor per lattice (TMA maps, constants, buffers, step count) and the tile list
-// of each group; the order of the tiles is the schedule.  Runs of graph_steps steps are
-// captured once into a CUDA graph and replayed.
+// Many independent lattices advanced together, by group of lattices that share a storage mode,
+// boundary kind and EOS.  Eight steps or more go as runs, one launch per group for many steps
+// (launch_runs).  Fewer, or with a kernel chosen by lbm_batch_set_kernel: one launch of the many-lattice
+// kernel per step and group, over the group's tile list, whose order is the schedule; graph_steps
+// such steps are captured once into a CUDA graph and replayed.  The workspace holds a descriptor
+// per lattice (TMA maps, constants, buffers, step count) and the tile lists.
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -18,7 +19,14 @@ struct Group {
     int st;
     bool walls, lang, flow, var_rho;
     int64_t off, count;  // tiles [off, off + count) of the tile list
+    lbm::RunDims run;    // the kernel of a run of steps of the group (blocks_per_sm 0: it does not fit)
+    std::vector<int> members;  // largest first
 };
+
+// Runs of steps, see launch_runs.  Tiles per SM from which a lattice fills the GPU by itself.
+constexpr int kAloneTilesPerSm = 20, kAloneTilesPerSm16 = 10;
+// Tiles of a cohort for every tile that the launch stages at a time.
+constexpr double kCohortTiles = 1.6, kCohortTiles16 = 6.0;
 
 int64_t tiles_of(const lbm_handle* h) { return (int64_t)h->tiles_x * h->tiles_y; }
 
@@ -26,7 +34,7 @@ int64_t tiles_of(const lbm_handle* h) { return (int64_t)h->tiles_x * h->tiles_y;
 Group group_of(const lbm_handle* h) {
     const bool flow = h->prm.velocity == LBM_VELOCITY_SOLVED;
     return Group{h->prm.storage, h->prm.bc_y == LBM_BC_WALLS, flow && h->prm.eos == LBM_EOS_LANGMUIR, flow,
-                 flow && h->phys.var_rho != 0, 0, 0};
+                 flow && h->phys.var_rho != 0, 0, 0, {}, {}};
 }
 
 bool same_group(const Group& a, const Group& b) {
@@ -65,7 +73,8 @@ struct lbm_batch {
     int kernel;            // LBM_KERNEL_AUTO, LBM_KERNEL_TILE or LBM_KERNEL_PIPELINED
     int ws_blocks[5];      // resident warp-specialised CTAs per SM of each members' storage mode (0: none)
     int sms;
-    unsigned* d_ctr;
+    int plain;             // 1: every step is a launch per group, as in lbm_batch_autotune
+    unsigned* d_ctr;       // two tile counters, and that of a run
     int ctr_parity;
     int graph_end_parity;
 };
@@ -100,8 +109,16 @@ int build_tiles(lbm_batch* b) {
         if (a.var_rho != c.var_rho) return a.var_rho < c.var_rho;
         return a.walls != c.walls ? a.walls < c.walls : a.lang < c.lang;
     });
+    std::vector<int> by_size(n);
+    for (int k = 0; k < n; ++k) by_size[k] = k;
+    std::stable_sort(by_size.begin(), by_size.end(),
+                     [&](int a, int c) { return tiles_of(b->members[a]) > tiles_of(b->members[c]); });
     std::vector<uint2> tiles;
     for (Group& g : groups) {
+        if (lbm::prepare_batch_run(g.st, lbm::Variant{g.walls, g.lang, g.flow, g.var_rho}, &g.run) != cudaSuccess)
+            return fail(LBM_ECUDA, "kernel setup failed");
+        for (int k : by_size)
+            if (same_group(group_of(b->members[k]), g)) g.members.push_back(k);
         g.off = (int64_t)tiles.size();
         std::vector<int> mem;
         for (int k : order)
@@ -202,6 +219,113 @@ int launch_one(lbm_batch* b, int s) {
     return LBM_OK;
 }
 
+// Whether `n` steps go as runs: always the faster way but for a few steps, whose launch and counters cost
+// more than they save.
+bool takes_runs(const lbm_batch* b, int64_t n) {
+    if (b->plain || b->kernel != LBM_KERNEL_AUTO || n < 8) return false;
+    int64_t tiles = 0;
+    for (const lbm_handle* h : b->members) {
+        if (h->tiles_y > kRowCounters) return false;
+        tiles += tiles_of(h);
+    }
+    for (const Group& g : b->groups)
+        if (g.run.blocks_per_sm < 1) return false;
+    return tiles <= 1 << 24;
+}
+
+// Whether a member's tiles fill the GPU by themselves: it then advances by lbm_step, whose kernel reads
+// its constants as kernel parameters.  16-bit storage gains from that at 13 tiles per SM (64-lattice mix
+// FP16, from 10 / 14 tiles per SM on: 302 / 310 us per step), FP32 later (364 / 356).
+bool runs_alone(const lbm_batch* b, const lbm_handle* h) {
+    if (h->chosen) return false;  // lbm_step would launch the chosen kernel for every step
+    return tiles_of(h) >= (int64_t)(lbm::pair_is_16bit(h->prm.storage) ? kAloneTilesPerSm16 : kAloneTilesPerSm) * b->sms;
+}
+
+// n steps of a group as runs.  The large members go one by one; the others, largest first, are cut into
+// cohorts which one launch advances all steps one after the other (see batch_kernel_run).  A cohort
+// must hold more tiles than the CTAs have claimed, or they wait for the level before (FP32 64-lattice
+// mix, 0.8 / 1.2 / 1.6 / 2 / 3 tiles per staged tile: 367 / 361 / 360 / 364 / 373 us per step), and few
+// enough that its state stays in L2.  16-bit storage gains little from L2 and much from never waiting
+// (FP16 0.8 / 1.6 / 3 / 6: 402 / 324 / 304 / 302).  Measured, us per step, one launch per step / runs:
+// 64-lattice mix FP32 392 / 356, FP16 302 / 302; 16 lattices FP32 119 / 104, FP16 95 / 91; 5 lattices
+// FP32 12.5 / 9.2, 3 lattices FP16 15.0 / 12.3; 12 server jobs FP32 and FP16 168 / 146.
+int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
+    const int slots = b->sms * g.run.blocks_per_sm;
+    const bool pair16 = lbm::pair_is_16bit(g.st);
+    const int want = (int)((pair16 ? kCohortTiles16 : kCohortTiles) * slots * g.run.buffers);
+    const lbm::TileDims td = lbm::tile_dims(g.st);
+    size_t at = 0;
+    for (; at < g.members.size() && runs_alone(b, b->members[g.members[at]]); ++at) {  // (largest first)
+        lbm_handle* h = b->members[g.members[at]];
+        const int64_t before = h->launches;
+        const int rc = lbm_step(h, n);
+        if (rc) return rc;
+        b->launches += h->launches - before;
+    }
+    for (; at < g.members.size(); at += lbm::kRunMembers) {
+        lbm::RunManyArgs a;
+        std::memset(&a, 0, sizeof(a));
+        a.descs = b->d_desc;
+        a.members = (int)std::min<size_t>(lbm::kRunMembers, g.members.size() - at);
+        int64_t total = 0;
+        int first = 0, tiles = 0, before = -1;  // members [first, ..) of the cohort at hand and their tiles; the cohort before
+        auto close = [&](int from, int to) {
+            int sum = 0;
+            for (int k = from; k < to; ++k) {
+                a.m[k].first = (unsigned short)from;
+                a.m[k].end = (unsigned short)to;
+                a.m[k].start = sum;
+                sum += a.m[k].ntx * a.m[k].nty;
+            }
+            for (int k = from; k < to; ++k) a.m[k].tiles = sum;
+        };
+        for (int k = 0; k < a.members; ++k) {
+            const int idx = g.members[at + k];
+            const lbm_handle* h = b->members[idx];
+            lbm::RunMember& m = a.m[k];
+            // (a periodic last tile row of one cell row makes two tile rows of a tile's reach, see lbm_step)
+            const int reach = !g.walls && h->prm.ny % td.ty == 1 ? 2 : 1;
+            m.rows = reinterpret_cast<unsigned*>(h->partials) + kRowOffset;
+            m.desc = idx;
+            m.ntx = (unsigned short)h->tiles_x;
+            m.nty = (unsigned short)h->tiles_y;
+            m.flags = reach << 2;
+            a.reach = std::max(a.reach, reach);
+            tiles += (int)tiles_of(h);
+            total += tiles_of(h);
+            if (tiles >= want) {
+                close(first, k + 1);
+                before = first;
+                first = k + 1;
+                tiles = 0;
+            }
+        }
+        if (first < a.members) close(before >= 0 && 2 * tiles < want ? before : first, a.members);
+        a.ring = g.run.buffers;
+        a.ahead = 16;
+        // tiles of a claim: few keep a cohort's level together, many ask the lead warp for fewer rounds
+        // (1 / 2 / 4 / 8, us per step: FP32 5 lattices of 6 tiles per SM in all 10.6 / 9.1 / 11.0 / 15.0; FP16
+        // 3 lattices, 7 tiles per SM, 13.2 / 12.4 / 13.7 / 17.5; FP16 8 lattices, 15 per SM, 25.5 / 23.2 / 22.6 / 22.6)
+        a.batch = total <= 3LL * slots ? 1 : (!pair16 || total <= 10LL * slots ? 2 : (total <= 16LL * slots ? 4 : 8));
+        if (a.reach > 1) a.batch = std::min(a.batch, 4);  // eight lanes of the lead warp per tile
+        a.ctr = b->d_ctr + 2;
+        const int64_t most = std::max<int64_t>(64, (1LL << 20) / total);
+        for (int64_t done = 0; done < n; done += a.nsteps) {
+            a.nsteps = (int)std::min(n - done, most);
+            for (int k = 0; k < a.members; ++k) {
+                const lbm_handle* h = b->members[a.m[k].desc];
+                a.m[k].steps = h->steps + done;
+                a.m[k].flags = (a.m[k].flags & ~3) | (int)((h->cur + done) & 1) | (h->first && done == 0 ? 2 : 0);
+            }
+            cudaError_t e = lbm::launch_batch_run(g.st, a, lbm::Variant{g.walls, g.lang, g.flow, g.var_rho},
+                                                  (int)std::min<int64_t>(total, slots), b->stream);
+            if (e != cudaSuccess) return fail(LBM_ECUDA, "batch run launch: %s", cudaGetErrorString(e));
+            b->launches += 2;
+        }
+    }
+    return LBM_OK;
+}
+
 int launch_advance(lbm_batch* b, int n) {
     const int count = (int)b->members.size();
     lbm::batch_advance_kernel<<<(count + 127) / 128, 128, 0, b->stream>>>(b->d_desc, count, n);
@@ -298,6 +422,7 @@ int lbm_batch_create(int max_members, int64_t max_tiles, void* d_workspace, size
     b->kernel = LBM_KERNEL_AUTO;
     for (int& w : b->ws_blocks) w = 0;
     b->sms = 0;
+    b->plain = 0;
     b->ctr_parity = 0;
     b->graph_end_parity = 0;
     b->schedule = LBM_SCHED_LARGEST_FIRST;
@@ -365,8 +490,12 @@ int lbm_batch_step(lbm_batch* b, int64_t n) {
         if (!h->initialized) return fail(LBM_ESTATE, "a member has no state (lbm_init_fields first)");
     int rc = upload_descs(b);
     if (rc) return rc;
-    int64_t done = 0;
-    if (b->graph_steps > 0 && n >= b->graph_steps) {
+    const bool runs = takes_runs(b, n);
+    if (runs)
+        for (size_t k = 0; k < b->groups.size() && !rc; ++k) rc = launch_runs(b, b->groups[k], n);
+    if (rc) return rc;
+    int64_t done = runs ? n : 0;
+    if (!runs && b->graph_steps > 0 && n >= b->graph_steps) {
         if (!b->graph) {
             rc = build_graph(b);
             if (rc) return rc;
@@ -383,6 +512,7 @@ int lbm_batch_step(lbm_batch* b, int64_t n) {
     if (!rc && rem > 0) rc = launch_advance(b, rem);
     if (rc) return rc;
     for (lbm_handle* h : b->members) {
+        if (runs && runs_alone(b, h)) continue;  // lbm_step counted them
         h->steps += n;
         h->cur = (int)((h->cur + n) & 1);
         h->first = 0;
@@ -404,6 +534,7 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_
     LBM_CUDA(cudaEventCreate(&e1));
     int rc = LBM_OK;
     int best = -1;
+    b->plain = 1;  // the schedule orders the launches of single steps
     for (size_t c = 0; c < cands.size() && !rc; ++c) {
         if (cands[c].sched < 0) cands[c].sched = cands[best].sched;
         rc = lbm_batch_set_schedule(b, cands[c].sched, cands[c].k);
@@ -418,6 +549,7 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_
         cands[c].ms = ms / (float)trial;
         if (!rc && (best < 0 || cands[c].ms < cands[best].ms)) best = (int)c;
     }
+    b->plain = 0;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;

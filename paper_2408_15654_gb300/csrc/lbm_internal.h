@@ -23,6 +23,12 @@ struct Layout {
     size_t off_pops[2], off_hist[2], off_shist[2], shist_bytes, off_status, off_partials, total;
 };
 
+// Counters of a run of steps: the tile counter, then the row counters.  They share the reduction's
+// partial sums (work of one handle is ordered on its stream).
+constexpr int kRowOffset = 32, kRowCounters = 2016;
+static_assert((kRowOffset + kRowCounters) * sizeof(unsigned) <= lbm::kMaxPartials * sizeof(double),
+              "the counters fit the partial sums");
+
 }  // namespace lbm_host
 
 #define LBM_CUDA(call)                                                                                   \
@@ -57,4 +63,5 @@ struct lbm_handle {
     int initialized;
     int first;        // 1 until the first step after lbm_init_fields
     int64_t steps;
+    int64_t launches;  // step kernels launched for this lattice alone
 };

@@ -1594,7 +1594,25 @@ template <int ST, bool WALLS, bool LANGMUIR, int FLOW> constexpr auto pipe_kerne
     else return step_kernel_pipe2<ST, WALLS, LANGMUIR, FLOW>;
 }
 
-// ---- a run of steps of one lattice in one launch ----
+// Per-lattice descriptor of a batch, in device memory, written by the host between launches and
+// advanced by batch_advance_kernel.  Buffer `cur` holds the current state; `steps` steps were taken
+// since initialisation.  The part that the threads of a tile read (InstCore) comes first: the kernels
+// stage it, or its constants, in shared memory with one bulk copy.
+struct alignas(16) InstCore {
+    Phys p;
+    void* pops[2];
+    float2* hist[2];
+    float2* shist[2];  // mass-flux history (density ratio != 1), else null
+    unsigned* status;
+    long long steps;
+};
+struct alignas(128) InstDesc : InstCore {
+    CUtensorMap tm_fg[2], tm_h[2], tm_hist[2];
+    int cur;
+    int first;
+};
+
+// ---- a run of steps of one lattice, or of many, in one launch ----
 struct RunArgs {
     CUtensorMap tm_fg[2], tm_h[2], tm_hist[2];  // of each buffer
     Phys p;
@@ -1615,26 +1633,52 @@ struct RunArgs {
     unsigned* rows;           // tiles finished per tile row (zero at start)
 };
 
+// One lattice of a run of many.  The lattices of a run are cut into cohorts, members [first, end); all
+// steps of a cohort come before those of the next.
+struct RunMember {
+    unsigned* rows;             // tiles finished per tile row (zero at start)
+    long long steps;            // steps taken before this launch
+    int desc;                   // index of its descriptor
+    int start;                  // its first tile in a level of its cohort
+    int tiles;                  // tiles in a level of its cohort
+    unsigned short first, end;  // members of its cohort
+    unsigned short ntx, nty;    // its tiles
+    int flags;                  // buffer of the current state | 2 on the first step after initialisation | reach << 2
+};
+constexpr int kRunMembers = 96;
+struct RunManyArgs {
+    RunMember m[kRunMembers];
+    const InstDesc* descs;
+    int members, nsteps;
+    int reach, ring, ahead, batch;  // as in RunArgs; reach: the largest of the members'
+    unsigned* ctr;                  // tile counter (zero at start)
+};
+static_assert(sizeof(RunManyArgs) <= 4096, "kernel parameters");
+
 // Shape of the persistent CTA: NG compute groups of NT threads, each updating its own tile, NB tile
 // buffers that TMA fills ahead of them, and four more warps (lead, signal and two copy warps).
-template <int ST, int FLOW> struct RunShape {
+// MANY: each buffer also holds the constants and buffers of its tile's lattice.
+template <int ST, int FLOW, bool MANY = false> struct RunShape {
     using G = GeoOf<ST>;
     using S = Smem<ST>;
     static constexpr int WPG = G::NT / 32;
-    static constexpr int NG = cpt_of(ST) == 1 ? (FLOW == kFlowVarRho ? 2 : 3) : (FLOW == kFlowVarRho ? 3 : 4);
+    static constexpr int NG = cpt_of(ST) == 1 ? (FLOW == kFlowVarRho ? 2 : 3) : (MANY || FLOW == kFlowVarRho ? 3 : 4);
+    static constexpr int CORE_BYTES = MANY ? (int)sizeof(InstCore) : 0;
     static constexpr int THREADS = NG * G::NT + 128;
     static constexpr int STAGE = FLOW ? S::PP : S::H;
     static constexpr int PP_ALL = 2 * NG * S::PP_BYTES;  // two (phi, psi) tiles per group, used in turn
     static constexpr int MAX_SMEM = 227 * 1024;
-    static constexpr int NB_FIT = (MAX_SMEM - PP_ALL - 44 * 8 * NG) / STAGE;
-    static constexpr int NB = NB_FIT < 8 ? NB_FIT : 8;
     static constexpr int DB = 8;                     // queue entries per group, used in turn
     static constexpr int QN = NG * DB;
+    static constexpr int NB_FIT = (MAX_SMEM - PP_ALL - 44 * QN) / (STAGE + CORE_BYTES);
+    static constexpr int NB = NB_FIT < 8 ? NB_FIT : 8;
     static constexpr int PP = NB * STAGE;
-    static constexpr int QUEUE = PP + PP_ALL;        // int4 per entry: x0 (-1: stop), y0, source buffer | first << 1, seed
+    static constexpr int QUEUE = PP + PP_ALL;        // int4 per entry: x0 (-1: stop), y0, source buffer | first << 1 | member << 2, seed
     static constexpr int BAR = QUEUE + 16 * QN;      // queued, full and done barrier of each entry
     static constexpr int SIG = BAR + 24 * QN;        // int per entry: how often it was signalled
-    static constexpr int BYTES = SIG + 4 * QN;
+    static constexpr int CORE = SIG + 4 * QN;
+    static constexpr int BYTES = CORE + NB * CORE_BYTES;
+    static_assert(CORE % 16 == 0, "bulk copies start on 16-byte boundaries");
     static_assert(NB >= NG && NB <= DB, "a buffer per group; queue entries for every buffer in use");
     static_assert(BYTES <= MAX_SMEM, "shared memory of one CTA");
 };
@@ -1708,6 +1752,37 @@ struct RunWalk {
     }
 };
 
+// The order of a run of many lattices: cohort by cohort, in each one level after the other, in each
+// level the members' tiles row by row.  With a periodic y the rows of level s start s reach further
+// around the ring, as in RunWalk.
+struct RunManyWalk {
+    int i, level, m;  // tile within the level of the cohort, level, member (m == members: past the end)
+    __device__ __forceinline__ void start(const RunManyArgs& a, int k) {
+        level = m = 0;
+        i = k;
+        settle(a);
+    }
+    __device__ __forceinline__ void move(const RunManyArgs& a, int d) {
+        i += d;
+        settle(a);
+    }
+    __device__ __forceinline__ void settle(const RunManyArgs& a) {
+        while (m < a.members) {
+            const int tiles = a.m[m].tiles;
+            if (i >= tiles) {
+                i -= tiles;
+                const bool over = ++level == a.nsteps;
+                if (over) level = 0;
+                m = over ? a.m[m].end : a.m[m].first;
+            } else if (m + 1 < a.m[m].end && i >= a.m[m + 1].start) {
+                ++m;
+            } else {
+                break;
+            }
+        }
+    }
+};
+
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
@@ -1754,10 +1829,10 @@ constexpr unsigned kRowPollLimit = 1u << 23;  // polls of 0.1 us or more: the wa
 // the earliest tile can always run: with claimed positions whichever CTAs are resident, with fixed ones
 // while all are (such launches are cooperative).  Every wait is bounded; a copy lane that gives up
 // waits (bounded) for its copies.
-template <int ST, bool WALLS, bool LANGMUIR, int FLOW>
-__global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
-    step_kernel_run(const __grid_constant__ RunArgs a) {
-    using Sh = RunShape<ST, FLOW>;
+template <int ST, bool WALLS, bool LANGMUIR, int FLOW, typename Args>
+__device__ __forceinline__ void run_body(const Args& a) {
+    constexpr bool kMany = std::is_same_v<Args, RunManyArgs>;
+    using Sh = RunShape<ST, FLOW, kMany>;
     using S = Smem<ST>;
     using G = GeoOf<ST>;
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -1780,6 +1855,11 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
     cudaTriggerProgrammaticLaunchCompletion();
     cudaGridDependencySynchronize();
     const int ring = a.ring, ng = min(Sh::NG, ring);
+    auto flag_timeout = [&]() {
+        if constexpr (kMany)
+            for (int n = 0; n < a.members; ++n) atomicOr(a.descs[a.m[n].desc].status, kStatusTimeout);
+        else atomicOr(a.status, kStatusTimeout);
+    };
     const int warp = (int)threadIdx.x / 32, lane = (int)threadIdx.x % 32;
     // an index that runs around a ring, and the parity of its turn
     auto advance = [](int& i, uint32_t& parity, int n, int size) {
@@ -1805,11 +1885,11 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
         // ---- lead warp: `batch` tiles at a time.  `share` successive lanes hold one of them, four for a
         // reach of one and eight for two; each asks for the counter of one of the tile rows around
         // it, so one round trip tells of all. ----
-        const int total = a.nsteps * a.ntx * a.nty;
         const int share = a.reach > 1 ? 8 : 4;
         const int off = lane % share - a.reach, n_own = lane / share;
         const unsigned mine = (1u << share) - 1u;
-        const int step = a.ctr ? 1 : (int)gridDim.x;
+        const bool claims = kMany || a.ctr;
+        const int step = claims ? 1 : (int)gridDim.x;
         const unsigned by_ng = ng > 1 ? 0xFFFFFFFFu / (unsigned)ng + 1u : 0u;  // j / ng as a product
         auto turn_of = [&](int j, int& e) {  // entry of tile j, and how often it was filled before
             const int m = ng > 1 ? (int)__umulhi((unsigned)j, by_ng) : j;
@@ -1817,13 +1897,21 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
             return m / Sh::DB;
         };
         auto claim = [&]() { return lane == 0 ? (int)atomicAdd(a.ctr, (unsigned)a.batch) : 0; };
-        int pos = a.ctr ? __shfl_sync(0xffffffffu, claim(), 0) : (int)blockIdx.x;
-        RunWalk walk;
-        walk.start<WALLS>(a, pos + n_own * step);
-        const int dq = a.batch * step / a.ntx, dc = a.batch * step - dq * a.ntx;  // of a round with fixed positions
+        int pos = claims ? __shfl_sync(0xffffffffu, claim(), 0) : (int)blockIdx.x;
+        std::conditional_t<kMany, RunManyWalk, RunWalk> walk;
+        int dq = 0, dc = 0, total = 0;  // one lattice: of a round with fixed positions; tiles of all steps
+        if constexpr (kMany) {
+            walk.start(a, pos + n_own);
+        } else {
+            walk.template start<WALLS>(a, pos + n_own * step);
+            dq = a.batch * step / a.ntx, dc = a.batch * step - dq * a.ntx;
+            total = a.nsteps * a.ntx * a.nty;
+        }
         for (int j0 = 0, left = 1; left; j0 += a.batch) {
-            const int later = a.ctr ? claim() : 0;  // the next claim, early (lane 0)
-            const bool live = pos + n_own * step < total && n_own < a.batch;
+            const int later = claims ? claim() : 0;  // the next claim, early (lane 0)
+            bool live = n_own < a.batch;
+            if constexpr (kMany) live = live && walk.m < a.members;
+            else live = live && pos + n_own * step < total;
             const unsigned count = __popc(__ballot_sync(0xffffffffu, live)) / share;
             left = count == a.batch;  // else the order ends in this round: stop marks follow, one per group
             // the first lane of a tile queues it; the one past the last tile queues the stop marks
@@ -1831,15 +1919,34 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
             const int j = j0 + n_own;
             int4 entry = make_int4(-1, 0, 0, 0);
             bool open = true;  // this lane's row is complete
-            const unsigned* rows = a.rows;
-            const unsigned need = (unsigned)walk.level * (unsigned)a.ntx;
+            const unsigned* rows = nullptr;
+            unsigned need = 0u;
             if (live) {
-                entry = make_int4(walk.col * G::TX, walk.row * G::TY, ((a.cur + walk.level) & 1) | (walk.level == 0 && a.first ? 2 : 0),
-                                  Traits<ST>::kPair16 ? (int)step_seed(a.steps + walk.level) : 0);
-                open = walk.level == 0 || off > a.reach;
-                int r = walk.row + off;
-                if (WALLS) r = min(max(r, 0), a.nty - 1);
-                else if (r < 0 || r >= a.nty) r = (r + 2 * a.nty) % a.nty;
+                int ntx, nty, row, col, reach, flags, member = 0;
+                long long steps;
+                if constexpr (kMany) {
+                    const RunMember& q = a.m[walk.m];
+                    member = walk.m;
+                    ntx = q.ntx, nty = q.nty, reach = q.flags >> 2, flags = q.flags & 3;
+                    rows = q.rows;
+                    steps = q.steps;
+                    row = (walk.i - q.start) / ntx;
+                    col = walk.i - q.start - row * ntx;
+                    if (!WALLS) row = (int)((row + (long long)walk.level * reach) % nty);
+                } else {
+                    ntx = a.ntx, nty = a.nty, reach = a.reach, flags = a.cur | (a.first ? 2 : 0);
+                    rows = a.rows;
+                    steps = a.steps;
+                    row = walk.row, col = walk.col;
+                }
+                need = (unsigned)walk.level * (unsigned)ntx;
+                entry = make_int4(col * G::TX, row * G::TY,
+                                  ((flags + walk.level) & 1) | (walk.level == 0 ? flags & 2 : 0) | (kMany ? member << 2 : 0),
+                                  Traits<ST>::kPair16 ? (int)step_seed(steps + walk.level) : 0);
+                open = walk.level == 0 || off > reach || (kMany && off < -reach);
+                int r = row + off;
+                if (WALLS) r = min(max(r, 0), nty - 1);
+                else if (r < 0 || r >= nty) r = (r + 2 * nty) % nty;
                 rows += r;
             }
             // queue each tile as soon as its rows and a queue entry are ready
@@ -1860,19 +1967,20 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
                     }
                 }
                 if (it == kRowPollLimit) {
-                    if (lane == 0) atomicOr(a.status, kStatusTimeout);
+                    if (lane == 0) flag_timeout();
                     return;
                 }
             }
             if (!left) return;
-            if (a.ctr) {
-                const int was = pos;
-                pos = __shfl_sync(0xffffffffu, later, 0);
+            const int was = pos;
+            pos = claims ? __shfl_sync(0xffffffffu, later, 0) : pos + a.batch * step;
+            if constexpr (kMany) {
+                walk.move(a, pos - was);
+            } else if (claims) {
                 const int q = (pos - was) / a.ntx;
-                walk.move<WALLS>(a, q, pos - was - q * a.ntx);
+                walk.template move<WALLS>(a, q, pos - was - q * a.ntx);
             } else {
-                pos += a.batch * step;
-                walk.move<WALLS>(a, dq, dc);
+                walk.template move<WALLS>(a, dq, dc);
             }
         }
         return;
@@ -1898,7 +2006,7 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
                 if (ok) last.next(ng);
             }
             if (!ok) {
-                atomicOr(a.status, kStatusTimeout);
+                flag_timeout();
                 for (; last.index() != tile.index(); last.next(ng)) mbar_wait_bounded(&full[last.index()], last.parity);
                 return;
             }
@@ -1906,12 +2014,22 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
             asm volatile("fence.proxy.async.global;\n" ::: "memory");
             const int src = e.z & 1;
             unsigned char* stage = sm + b * Sh::STAGE;
+            const CUtensorMap *fg, *hm, *hist;
+            if constexpr (kMany) {
+                const InstDesc& d = a.descs[a.m[e.z >> 2].desc];
+                fg = &d.tm_fg[src], hm = &d.tm_h[src], hist = &d.tm_hist[src];
+            } else {
+                fg = &a.tm_fg[src], hm = &a.tm_h[src], hist = &a.tm_hist[src];
+            }
             if (first) {
                 // (the other half may have begun to arrive: the barrier waits for this arrival)
-                mbar_expect_tx(&full[tile.index()], FLOW ? S::TX_BYTES : S::TX_BYTES_NOH);
-                issue_boxes<ST, FLOW, 0, 2>(stage, &a.tm_fg[src], &a.tm_h[src], &a.tm_hist[src], e.x, e.y, &full[tile.index()]);
+                mbar_expect_tx(&full[tile.index()], (FLOW ? S::TX_BYTES : S::TX_BYTES_NOH) + Sh::CORE_BYTES);
+                if constexpr (kMany)
+                    bulk_copy_g2s(sm + Sh::CORE + b * Sh::CORE_BYTES, &a.descs[a.m[e.z >> 2].desc], Sh::CORE_BYTES,
+                                  &full[tile.index()]);
+                issue_boxes<ST, FLOW, 0, 2>(stage, fg, hm, hist, e.x, e.y, &full[tile.index()]);
             } else {
-                issue_boxes<ST, FLOW, 1, 2>(stage, &a.tm_fg[src], &a.tm_h[src], &a.tm_hist[src], e.x, e.y, &full[tile.index()]);
+                issue_boxes<ST, FLOW, 1, 2>(stage, fg, hm, hist, e.x, e.y, &full[tile.index()]);
             }
         }
     }
@@ -1922,17 +2040,18 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
         bool live = lane < ng;
         uint32_t parity = 0u;
         for (unsigned idle = 0; __any_sync(0xffffffffu, live);) {
-            int row = -1;
+            unsigned* row = nullptr;
             const bool moved = live && mbar_test(&done[own + d], parity);
             if (moved) {
                 const int4 e = queue[own + d];
                 live = e.x >= 0;
-                row = live ? e.y / G::TY : -1;
+                if constexpr (kMany) row = live ? a.m[e.z >> 2].rows + e.y / G::TY : nullptr;
+                else row = live ? a.rows + e.y / G::TY : nullptr;
             }
             if (__any_sync(0xffffffffu, moved)) {
                 idle = 0;
                 // the tile's stores, which the group's arrivals tell of, before the count
-                if (row >= 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(a.rows + row) : "memory");
+                if (row) asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(row) : "memory");
                 if (moved) {
                     st_shared_release(&signalled[own + d], turns + 1);
                     if (++d == Sh::DB) {
@@ -1943,7 +2062,7 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
                 }
             } else {
                 if (++idle == kRowPollLimit) {
-                    if (lane == 0) atomicOr(a.status, kStatusTimeout);
+                    if (lane == 0) flag_timeout();
                     return;
                 }
                 __nanosleep(40);
@@ -1970,21 +2089,35 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
             else if (lane == 0) mbar_arrive(&done[at]);
             return;
         }
+        if constexpr (kMany) {
+            // a copy that did not come in time: no constants to read, so meet the barriers of step_tile here
+            if (__any_sync(0xffffffffu, late)) {
+                if (lane == 0) flag_timeout();
+                compute_sync_or<G::NT>(1 + g, true);
+                if (lane == 0) mbar_wait_bounded(mbar, parity);
+                compute_sync<G::NT>(1 + g);
+                return;
+            }
+        }
         const int src = e.z & 1;
+        const auto& io_of = [&]() -> const auto& {
+            if constexpr (kMany) return *reinterpret_cast<const InstCore*>(sm + Sh::CORE + b * Sh::CORE_BYTES);
+            else return a;
+        }();
         TileIO io;
         io.src = nullptr;
         io.hist_src = nullptr;
-        io.dst = src ? a.pops[0] : a.pops[1];
-        io.hist_dst = src ? a.hist[0] : a.hist[1];
-        io.shist_src = src ? a.shist[1] : a.shist[0];
-        io.shist_dst = src ? a.shist[0] : a.shist[1];
-        io.status = a.status;
+        io.dst = src ? io_of.pops[0] : io_of.pops[1];
+        io.hist_dst = src ? io_of.hist[0] : io_of.hist[1];
+        io.shist_src = src ? io_of.shist[1] : io_of.shist[0];
+        io.shist_dst = src ? io_of.shist[0] : io_of.shist[1];
+        io.status = io_of.status;
         io.out[0] = io.out[1] = io.out[2] = io.out[3] = io.out[4] = nullptr;
         io.seed = (unsigned)e.w;
-        io.first = e.z >> 1;
+        io.first = e.z >> 1 & 1;
         float2* PP = reinterpret_cast<float2*>(sm + Sh::PP + (2 * g + (int)(m & 1u)) * S::PP_BYTES);
-        if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(a.p, io, sm + b * Sh::STAGE, PP, mbar, parity, e.x, e.y, t,
-                                                                  1 + g, late))
+        if (step_tile_any<ST, WALLS, LANGMUIR, kStep, FLOW, true>(io_of.p, io, sm + b * Sh::STAGE, PP, mbar, parity, e.x, e.y,
+                                                                  t, 1 + g, late))
             return;  // uniform (decided by the OR barrier inside)
         __syncwarp();
         if (lane == 0) mbar_arrive(&done[at]);
@@ -1992,22 +2125,28 @@ __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1)
     }
 }
 
-// ---- many lattices in one launch ----
-// Per-lattice descriptor, in device memory, written by the host between launches and advanced by
-// batch_advance_kernel.  Buffer `cur` holds the current state; `steps` steps were taken since
-// initialisation.
-struct alignas(128) InstDesc {
-    CUtensorMap tm_fg[2], tm_h[2], tm_hist[2];
-    Phys p;
-    void* pops[2];
-    float2* hist[2];
-    float2* shist[2];  // mass-flux history (density ratio != 1), else null
-    unsigned* status;
-    long long steps;
-    int cur;
-    int first;
-};
+template <int ST, bool WALLS, bool LANGMUIR, int FLOW>
+__global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1) step_kernel_run(const __grid_constant__ RunArgs a) {
+    run_body<ST, WALLS, LANGMUIR, FLOW>(a);
+}
+// The same for many lattices.  A tile's lattice constants come with its boxes (one more bulk copy), which
+// costs registers: with two cells per thread three groups of 128 registers do better than four of 96,
+// which spill (64-lattice mix FP16: 321 / 366 us per step).  What bounds it: with FP32 storage and
+// the state in L2 the compute groups wait for tiles 40 % of the time and issue in 48 % of the cycles (five
+// buffers fill the SM: with four the mix takes 414 us instead of 373), with 16-bit storage the latency
+// of the cell update at twelve compute warps per SM.
+template <int ST, bool WALLS, bool LANGMUIR, int FLOW>
+__global__ void __launch_bounds__(RunShape<ST, FLOW, true>::THREADS, 1)
+    batch_kernel_run(const __grid_constant__ RunManyArgs a) {
+    run_body<ST, WALLS, LANGMUIR, FLOW>(a);
+}
+// Zero the counters of a run of many lattices: block k those of member k.
+static __global__ void batch_run_reset_kernel(const __grid_constant__ RunManyArgs a) {
+    for (int r = threadIdx.x; r < a.m[blockIdx.x].nty; r += blockDim.x) a.m[blockIdx.x].rows[r] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.ctr = 0u;
+}
 
+// ---- many lattices, one launch per step ----
 // Launch s (0-based) of a sequence that started from the descriptors' state; each CTA owns the
 // tile tiles[blockIdx.x] = (lattice, tile column | tile row << 16).
 struct BatchArgs {

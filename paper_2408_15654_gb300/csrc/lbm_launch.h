@@ -1,6 +1,5 @@
-// Launch helpers of the step kernels, one translation unit per storage mode
-// (step_fp32.cu, step_fp16.cu, step_bf16.cu, step_fp16fg.cu, step_bf16fg.cu) so that the
-// instances compile in parallel.  Each storage mode has ten kernel variants: walls or periodic y
+// Launch helpers of the step kernels, two translation units per storage mode (step_fp32.cu,
+// batch_fp32.cu, step_fp16.cu, ..) so that the instances compile in parallel.  Each storage mode has ten kernel variants: walls or periodic y
 // and Langmuir or linear EOS with the flow solved at uniform density or with a density ratio, and
 // walls or periodic y with the velocity prescribed (no flow populations; the EOS is unused).
 #pragma once
@@ -123,15 +122,38 @@ template <int ST> cudaError_t prepare_run_impl(const Variant& v, RunDims* d) {
     });
 }
 
-// Opt every variant of storage mode ST into its dynamic shared memory; resident CTAs per SM of the
-// one-tile kernels (the minimum over the variants) and of the pipelined kernel of variant `use`
-// (its register use differs between the variants: a minimum would hold every variant to the
-// density-ratio update's 128 registers).
+// A run of steps of many lattices of one variant, positions claimed from a.ctr, which together with the
+// members' counters is zeroed before.
+template <int ST>
+cudaError_t launch_batch_run_impl(const RunManyArgs& a, const Variant& v, int ctas, cudaStream_t stream) {
+    batch_run_reset_kernel<<<a.members, 128, 0, stream>>>(a);
+    cudaError_t r = cudaGetLastError();
+    if (r != cudaSuccess) return r;
+    return dispatch_variant(v, [&]<bool W, bool L, int F>() {
+        using Sh = RunShape<ST, F, true>;
+        batch_kernel_run<ST, W, L, F><<<ctas, Sh::THREADS, Sh::BYTES, stream>>>(a);
+        return cudaGetLastError();
+    });
+}
+
+// Opt the run kernel of many lattices of variant v into its shared memory and describe it.
+template <int ST> cudaError_t prepare_batch_run_impl(const Variant& v, RunDims* d) {
+    return dispatch_variant(v, [&]<bool W, bool L, int F>() {
+        using Sh = RunShape<ST, F, true>;
+        d->buffers = Sh::NB;
+        auto k = batch_kernel_run<ST, W, L, F>;
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Sh::BYTES);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&d->blocks_per_sm, k, Sh::THREADS, Sh::BYTES);
+        return e;
+    });
+}
+
+// Opt the step kernels of variant `use` into their dynamic shared memory; resident CTAs per SM of the
+// one-tile kernels (the smaller of the two) and of the pipelined kernel.
 template <int ST>
 cudaError_t prepare_step_impl(const Variant& use, int* blocks_per_sm, int* pipe_blocks_per_sm) {
-    int tile = 1 << 30, pipe = 0;
-    auto one = [&]<bool W, bool L, int F>() -> cudaError_t {
-        int b = 0;
+    return dispatch_variant(use, [&]<bool W, bool L, int F>() -> cudaError_t {
+        int b0 = 0, b1 = 0;
         auto k0 = step_kernel<ST, W, L, kStep, F>;
         auto k1 = step_kernel<ST, W, L, kMoments, F>;
         auto kp = pipe_kernel<ST, W, L, F>();
@@ -139,22 +161,13 @@ cudaError_t prepare_step_impl(const Variant& use, int* blocks_per_sm, int* pipe_
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<ST>::BYTES);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<ST>::BYTES_PIPE);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k0, GeoOf<ST>::NT, Smem<ST>::BYTES);
-        tile = b < tile ? b : tile;
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k1, GeoOf<ST>::NT, Smem<ST>::BYTES);
-        tile = b < tile ? b : tile;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b0, k0, GeoOf<ST>::NT, Smem<ST>::BYTES);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b1, k1, GeoOf<ST>::NT, Smem<ST>::BYTES);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(pipe_blocks_per_sm, kp, nt_pipe<ST>(), Smem<ST>::BYTES_PIPE);
+        *blocks_per_sm = b0 < b1 ? b0 : b1;
         return e;
-    };
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < kVariants && e == cudaSuccess; ++k) e = dispatch_variant(variant_of(k), one);
-    if (e == cudaSuccess)
-        e = dispatch_variant(use, [&]<bool W, bool L, int F>() {
-            return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pipe, pipe_kernel<ST, W, L, F>(), nt_pipe<ST>(),
-                                                                 Smem<ST>::BYTES_PIPE);
-        });
-    *blocks_per_sm = tile;
-    *pipe_blocks_per_sm = pipe;
-    return e;
+    });
 }
 
 // One launch of the many-lattice kernel over `ntiles` tiles (all lattices of one variant): one CTA
@@ -204,6 +217,8 @@ cudaError_t launch_run(int st, const RunArgs& a, const Variant& v, int ctas, cud
 cudaError_t prepare_run(int st, const Variant& v, RunDims* d);
 cudaError_t launch_batch(int st, const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s);
 cudaError_t prepare_batch(int st, int* ws_blocks_per_sm);
+cudaError_t launch_batch_run(int st, const RunManyArgs& a, const Variant& v, int ctas, cudaStream_t s);
+cudaError_t prepare_batch_run(int st, const Variant& v, RunDims* d);
 
 #define LBM_DECLARE_STORAGE(name)                                                                                  \
     cudaError_t launch_step_##name(const StepArgs& a, int mode, const Variant& v, dim3 grid, int pipe,              \
@@ -212,7 +227,9 @@ cudaError_t prepare_batch(int st, int* ws_blocks_per_sm);
     cudaError_t launch_run_##name(const RunArgs& a, const Variant& v, int ctas, cudaStream_t s);                    \
     cudaError_t prepare_run_##name(const Variant& v, RunDims* d);                                                   \
     cudaError_t launch_batch_##name(const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s);         \
-    cudaError_t prepare_batch_##name(int* ws_blocks_per_sm);
+    cudaError_t prepare_batch_##name(int* ws_blocks_per_sm);                                                        \
+    cudaError_t launch_batch_run_##name(const RunManyArgs& a, const Variant& v, int ctas, cudaStream_t s);          \
+    cudaError_t prepare_batch_run_##name(const Variant& v, RunDims* d);
 LBM_DECLARE_STORAGE(fp32)
 LBM_DECLARE_STORAGE(fp16)
 LBM_DECLARE_STORAGE(bf16)
@@ -232,10 +249,17 @@ LBM_DECLARE_STORAGE(bf16fg)
     cudaError_t launch_run_##name(const RunArgs& a, const Variant& v, int ctas, cudaStream_t s) {                   \
         return launch_run_impl<ST>(a, v, ctas, s);                                                                 \
     }                                                                                                              \
-    cudaError_t prepare_run_##name(const Variant& v, RunDims* d) { return prepare_run_impl<ST>(v, d); }             \
+    cudaError_t prepare_run_##name(const Variant& v, RunDims* d) { return prepare_run_impl<ST>(v, d); }
+
+// Body of a per-storage translation unit of the batch kernels.
+#define LBM_DEFINE_BATCH(name, ST)                                                                                 \
     cudaError_t launch_batch_##name(const BatchArgs& b, const Variant& v, unsigned ntiles, cudaStream_t s) {        \
         return launch_batch_impl<ST>(b, v, ntiles, s);                                                            \
     }                                                                                                              \
-    cudaError_t prepare_batch_##name(int* ws_blocks_per_sm) { return prepare_batch_impl<ST>(ws_blocks_per_sm); }
+    cudaError_t prepare_batch_##name(int* ws_blocks_per_sm) { return prepare_batch_impl<ST>(ws_blocks_per_sm); }     \
+    cudaError_t launch_batch_run_##name(const RunManyArgs& a, const Variant& v, int ctas, cudaStream_t s) {         \
+        return launch_batch_run_impl<ST>(a, v, ctas, s);                                                           \
+    }                                                                                                              \
+    cudaError_t prepare_batch_run_##name(const Variant& v, RunDims* d) { return prepare_batch_run_impl<ST>(v, d); }
 
 }  // namespace lbm

@@ -56,6 +56,26 @@ cudaError_t launch_batch(int st, const BatchArgs& b, const Variant& v, unsigned 
     }
 }
 
+cudaError_t launch_batch_run(int st, const RunManyArgs& a, const Variant& v, int ctas, cudaStream_t s) {
+    switch (st) {
+        case kFP16: return launch_batch_run_fp16(a, v, ctas, s);
+        case kBF16: return launch_batch_run_bf16(a, v, ctas, s);
+        case kFP16FG: return launch_batch_run_fp16fg(a, v, ctas, s);
+        case kBF16FG: return launch_batch_run_bf16fg(a, v, ctas, s);
+        default: return launch_batch_run_fp32(a, v, ctas, s);
+    }
+}
+
+cudaError_t prepare_batch_run(int st, const Variant& v, RunDims* d) {
+    switch (st) {
+        case kFP16: return prepare_batch_run_fp16(v, d);
+        case kBF16: return prepare_batch_run_bf16(v, d);
+        case kFP16FG: return prepare_batch_run_fp16fg(v, d);
+        case kBF16FG: return prepare_batch_run_bf16fg(v, d);
+        default: return prepare_batch_run_fp32(v, d);
+    }
+}
+
 cudaError_t prepare_batch(int st, int* ws_blocks_per_sm) {
     switch (st) {
         case kFP16: return prepare_batch_fp16(ws_blocks_per_sm);

@@ -377,7 +377,8 @@ def lbm_batch_destroy(b: int):
 
 
 class Batch:
-    """Many ``Lattice`` objects advanced together (one launch per step and member group).
+    """Many ``Lattice`` objects advanced together (runs of many steps in one launch per member group, or
+    one launch per step and group).
 
     All members must use the batch's stream.  ``capacity`` bounds the member count and
     ``max_tiles`` the total tile count (default: exactly what ``lattices`` need)."""
