@@ -358,12 +358,16 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
         }
     }
     // Claimed tiles balance the SMs, whose shares of the memory differ (2048 x 1024, one level at a
-    // time, fixed / claimed: FP32 78.3 / 68.8, FP16 47.0 / 43.3); a claim takes four, since the lead
+    // time, fixed / claimed: FP32 78.3 / 68.8, FP16 47.0 / 43.3); a claim takes several, since the lead
     // warp's round takes 2 us.  Up to about ten tiles per SM fixed positions do better (608 x 512 FP32
     // 8.3 / 8.7, 128 x 128 4.0 / 5.2), and so do several levels at a time, which claims ahead of their
-    // turn would hold apart (67.1 / 69.4).
+    // turn would hold apart (67.1 / 69.4).  Tiles of a claim: two keep successive levels closer together,
+    // which FP32 gains from and small grids need; eight save rounds of the lead warp where the levels are
+    // long (us per step with 2 / 4 / 8: FP32 1024 x 512 16.0 / 16.5 / 18.0, 1024^2 34.4 / 35.0 / 35.5; FP16
+    // 768^2 14.0 / 14.1 / 15.2, 1024^2 23.6 / 22.3 / 22.2, 2048 x 1024 48.1 / 43.1 / 42.8).
     const bool fixed = a.depth > 1 || tiles <= 10LL * slots;
-    a.batch = !fixed ? 4 : (tiles <= 4LL * slots ? 1 : 2);
+    if (fixed) a.batch = tiles <= 4LL * slots ? 1 : 2;
+    else a.batch = !pair16 || tiles <= 16LL * slots ? 2 : (tiles <= 50LL * slots || a.reach > 1 ? 4 : 8);
     const int ctas = (int)std::min<long long>(tiles, slots);
     unsigned* c = reinterpret_cast<unsigned*>(h->partials);
     LBM_CUDA(cudaMemsetAsync(c, 0, (size_t)(kRowOffset + a.nty) * sizeof(unsigned), h->stream));
