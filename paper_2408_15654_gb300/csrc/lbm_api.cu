@@ -380,23 +380,24 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     return LBM_OK;
 }
 
-// FP64 sum of phi (lane 0) or psi (lane 1) of a population buffer into partials[0..blocks),
-// then partials[blocks] ... written to *dres.
+// FP64 sum of phi (lane 0) or psi (lane 1) of a population buffer into partials[0..blocks), then
+// their sum to *dres: by the same launch with a counter `finished`, else by another one.
 int launch_reduce(int st, const void* pops, int lane, bool pulled, int nx, int ny, int pitch, size_t plane, long long org,
                   const lbm::Phys& ph,
-                  int blocks, double* partials, double* dres, cudaStream_t stream) {
+                  int blocks, double* partials, unsigned* finished, double* dres, cudaStream_t stream) {
     // the pair planes of the FG modes are stored like those of the all-16-bit modes
     const long long pl = (long long)plane;
     if (st == LBM_STORE_FP16 || st == LBM_STORE_FP16_FG)
         lbm::reduce_partial_kernel<lbm::kFP16><<<blocks, lbm::kReduceThreads, 0, stream>>>(pops, lane, pulled, nx, ny,
-                                                                                           pitch, pl, org, ph, partials);
+                                                                                           pitch, pl, org, ph, partials, finished, dres);
     else if (st == LBM_STORE_BF16 || st == LBM_STORE_BF16_FG)
         lbm::reduce_partial_kernel<lbm::kBF16><<<blocks, lbm::kReduceThreads, 0, stream>>>(pops, lane, pulled, nx, ny,
-                                                                                           pitch, pl, org, ph, partials);
+                                                                                           pitch, pl, org, ph, partials, finished, dres);
     else
         lbm::reduce_partial_kernel<lbm::kFP32><<<blocks, lbm::kReduceThreads, 0, stream>>>(pops, lane, pulled, nx, ny,
-                                                                                           pitch, pl, org, ph, partials);
+                                                                                           pitch, pl, org, ph, partials, finished, dres);
     LBM_CUDA(cudaGetLastError());
+    if (finished) return LBM_OK;
     lbm::reduce_final_kernel<<<1, lbm::kReduceThreads, 0, stream>>>(partials, blocks, dres);
     LBM_CUDA(cudaGetLastError());
     return LBM_OK;
@@ -518,7 +519,7 @@ int lbm_reduce_noalloc(const void* d_pops, int nx, int ny, int what, void* cuda_
     lbm::Phys ph;
     std::memset(&ph, 0, sizeof(ph));
     rc = launch_reduce(LBM_STORE_FP32, d_pops, what == LBM_SUM_PSI ? 1 : 0, false, nx, ny, pitch, plane, org, ph, ny,
-                       scratch, scratch + LBM_NOALLOC_MAX_ROWS, stream);
+                       scratch, nullptr, scratch + LBM_NOALLOC_MAX_ROWS, stream);
     if (rc) return rc;
     LBM_CUDA(cudaMemcpyAsync(out, scratch + LBM_NOALLOC_MAX_ROWS, sizeof(double), cudaMemcpyDeviceToHost, stream));
     LBM_CUDA(cudaStreamSynchronize(stream));
@@ -733,16 +734,22 @@ int lbm_reduce(lbm_handle* h, int what, double* out) {
     if (what != LBM_SUM_PHI && what != LBM_SUM_PSI) return fail(LBM_EINVAL, "bad reduction selector");
     if (!out) return fail(LBM_EINVAL, "out is NULL");
     const int blocks = h->prm.ny < lbm::kMaxPartials ? h->prm.ny : lbm::kMaxPartials;
-    double* dres = h->partials + lbm::kMaxPartials;
+    // the status word, the counter and the sum lie side by side and come back in one copy
+    struct Result {
+        unsigned status, pad, tile_ctr[2], finished, pad2;
+        double sum;
+    } r;
+    static_assert(offsetof(Result, sum) == 24 && sizeof(Result) <= kAlign, "the status region holds the result");
+    Result* d = reinterpret_cast<Result*>(h->status);
     // before the first step the buffer is staged for the first pull (see reduce_partial_kernel)
     int rc = launch_reduce(h->prm.storage, h->pops[h->cur], what == LBM_SUM_PSI ? 1 : 0, h->first != 0, h->prm.nx,
-                           h->prm.ny, h->L.pitch, h->L.plane, h->phys.org, h->phys, blocks, h->partials, dres, h->stream);
+                           h->prm.ny, h->L.pitch, h->L.plane, h->phys.org, h->phys, blocks, h->partials, &d->finished, &d->sum,
+                           h->stream);
     if (rc) return rc;
-    LBM_CUDA(cudaMemcpyAsync(out, dres, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    unsigned st = 0;
-    rc = read_status(h, &st);
-    if (rc) return rc;
-    return status_code(st);
+    LBM_CUDA(cudaMemcpyAsync(&r, d, sizeof(r), cudaMemcpyDeviceToHost, h->stream));
+    LBM_CUDA(cudaStreamSynchronize(h->stream));
+    *out = r.sum;
+    return status_code(r.status);
 }
 
 int lbm_status(lbm_handle* h) {

@@ -2485,25 +2485,37 @@ __device__ __forceinline__ double block_sum(double v, double* smem) {
     return v;
 }
 
+__device__ __forceinline__ double sum_partials(const double* partials, int n, double* smem) {
+    double acc = 0.0;
+    for (int k = threadIdx.x; k < n; k += blockDim.x) acc += __ldcg(partials + k);
+    return block_sum(acc, smem);
+}
+
 // lane 0 sums f (phi), lane 1 sums g (psi); 16-bit storage is decoded to its value first;
-// pulled: sum the values at x - c_i (the state before the first step) instead of the own slots
+// pulled: sum the values at x - c_i (the state before the first step) instead of the own slots.
+// With a counter (zero between launches) the block that finishes last also adds up the partial sums,
+// in the order of reduce_final_kernel, which saves a launch (one step, the fields and both sums at
+// 256 x 256, with one copy back per sum instead of two: 99 -> 79 us).
 template <int ST>
 __global__ void __launch_bounds__(kReduceThreads) reduce_partial_kernel(const void* __restrict__ pops, int lane,
                                                                         int pulled, int nx, int ny, int pitch,
                                                                         long long plane,
                                                                         long long org, Phys p,
-                                                                        double* __restrict__ partials) {
+                                                                        double* partials, unsigned* finished, double* out) {
     using T = Traits<ST>;
     using P = typename T::P;
     __shared__ double smem[32];
+    __shared__ bool last;
     const P* pairs = static_cast<const P*>(pops);
     double acc = 0.0;
     // block b owns rows b, b + gridDim.x, ...; threads stride over (pair plane, x), counted in 64
     // bits (9 nx exceeds the int range for rows wider than 2^31 / 9 cells)
     const long long nk = (long long)kPairs * nx;
     for (int y = blockIdx.x; y < ny; y += gridDim.x) {
-        for (long long k = threadIdx.x; k < nk; k += blockDim.x) {
-            const int i = (int)(k / nx), x = (int)(k - (long long)i * nx);
+        long long x_ = threadIdx.x;  // k = i nx + x
+        for (long long k = threadIdx.x, i_ = 0; k < nk; k += blockDim.x, x_ += blockDim.x) {
+            for (; x_ >= nx; x_ -= nx) ++i_;
+            const int i = (int)i_, x = (int)x_;
             const int sx = pulled ? x - cx(i) : x, sy = pulled ? y - cy(i) : y;
             const float2 v = raw2(pairs[(size_t)i * plane + (size_t)(org + (long long)sy * pitch + sx)]);
             if constexpr (!T::kPair16) {
@@ -2515,7 +2527,19 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_partial_kernel(const vo
         }
     }
     acc = block_sum(acc, smem);
-    if (threadIdx.x == 0) partials[blockIdx.x] = acc;
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = acc;
+        if (finished) {
+            __threadfence();
+            last = atomicInc(finished, gridDim.x - 1) == gridDim.x - 1;  // back to zero with the last block
+            __threadfence();
+        }
+    }
+    if (!finished) return;
+    __syncthreads();
+    if (!last) return;
+    acc = sum_partials(partials, (int)gridDim.x, smem);
+    if (threadIdx.x == 0) *out = acc;
 }
 
 // Failure-detection self-test: one warp waits, with the bounded wait of the step kernels, on an
@@ -2536,9 +2560,7 @@ static __global__ void selftest_wait_kernel(unsigned* __restrict__ status) {
 static __global__ void __launch_bounds__(kReduceThreads) reduce_final_kernel(const double* __restrict__ partials, int n,
                                                                       double* __restrict__ out) {
     __shared__ double smem[32];
-    double acc = 0.0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) acc += partials[k];
-    acc = block_sum(acc, smem);
+    const double acc = sum_partials(partials, n, smem);
     if (threadIdx.x == 0) *out = acc;
 }
 
