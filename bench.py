@@ -4,8 +4,8 @@
 
 Workload: the sheared drop on a 2048 x 1024 grid (walls at +/-0.01, R = 160, Re = 1, Ca = 0.2,
 Langmuir EOS E0 = 0.2, psi0 = 0.3), populations stored in FP32, synthetic seeded fields.  A step is
-one lbm_step(1): one launch of the fused collide-stream kernel over the whole grid.  The metric is
-MLUPS (million lattice updates per second; one update advances f, g and h of one cell).  The
+one fused collide-stream update of the whole grid; a window is one lbm_step(K), which launches a
+persistent kernel for up to 128 steps at a time.  The metric is MLUPS (million lattice updates per second; one update advances f, g and h of one cell).  The
 populations (436 MB) exceed the 129 MB L2, so no flush is needed between steps.
 
 Timing: after W untimed steps, windows of exactly K steps are timed with CUDA events on the
@@ -234,6 +234,19 @@ def timed_windows(torch, stream, advance, k: int, min_s: float = None, max_windo
     return statistics.median(times), len(times)
 
 
+def step_launches(n: int, nx: int, ny: int, sms: int, pair16: bool = False) -> int:
+    """Step kernels that one lbm_step(n) launches: runs of max(64, 2^20 / tiles) steps, and one launch per
+    step for a few steps or for 16-bit grids of one to three tiles per SM."""
+    tiles = -(-nx // 32) * -(-ny // 8)
+    launches = 0
+    while n > 0:
+        runs = n >= (4 if tiles > 8 * sms else 8) and not (pair16 and sms < tiles <= 3 * sms)
+        took = min(n, max(64, (1 << 20) // tiles)) if runs else 1
+        n -= took
+        launches += 1
+    return launches
+
+
 def oracle_mlups(oracle, p, f, threads: int, budget_s: float, max_steps: int = 200):
     """The FP64 oracle on `threads` host threads: whole steps of one lattice (after 1 untimed step)
     until about budget_s seconds; returns (MLUPS, steps timed)."""
@@ -287,9 +300,9 @@ def cpu_baselines(budget_s: float = 4.0):
 
 
 def batch_leg(torch, lbm, W, storage: str, steps: int, alone_steps: int = 0):
-    """The 64-lattice mix (sizes 128^2 .. 1024x512, seed 0) advanced by one launch per step:
+    """The 64-lattice mix (sizes 128^2 .. 1024x512, seed 0) advanced by lbm_batch_step:
     autotuned schedule, then `steps` device-timed steps; optionally each lattice alone for
-    `alone_steps` steps (one lbm_step launch per lattice and step) for comparison."""
+    `alone_steps` steps (lbm_step on one lattice after the other) for comparison."""
     bstream = torch.cuda.Stream()
     inst = W.batch_instances(64, seed=0)
     lats = []
@@ -323,7 +336,9 @@ def batch_leg(torch, lbm, W, storage: str, steps: int, alone_steps: int = 0):
         a1.record(bstream)
         torch.cuda.synchronize()
         out["one_at_a_time"] = {"value": sig(cells * alone_steps / (a0.elapsed_time(a1) * 1e-3) / 1e6),
-                                "unit": "MLUPS", "steps": alone_steps, "gpu_launches": 64 * alone_steps}
+                                "unit": "MLUPS", "steps": alone_steps, "gpu_launches": sum(step_launches(alone_steps, g.nx, g.ny,
+                                                                  torch.cuda.get_device_properties(0).multi_processor_count,
+                                                                  storage != "fp32") for g in lats)}
     b.close()
     for g in lats:
         g.close()
@@ -500,6 +515,8 @@ def run_ours(args):
         raise RuntimeError(f"unstable state during the benchmark: {lbm.lbm_last_error()}")
     value = aggregate_mlups(cells, args.steps, world, ms_max)
     timed_steps = args.steps * nwin
+    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
+    window_launches = step_launches(args.steps, NX, NY, sms)
 
     # ---- the same workload with 16-bit population storage (FP32 arithmetic) ----
     half = {}
@@ -620,7 +637,7 @@ def run_ours(args):
             "e2e": {"value": e2e, "unit": "MLUPS", "h2d_bytes_per_step": io_bytes / args.steps,
                     "d2h_bytes_per_step": io_bytes / args.steps,
                     "job": f"lbm_init_fields(host) + lbm_step({args.steps}) + lbm_get_moments(host, all 5)"},
-            "gpu_launches": timed_steps,
+            "gpu_launches": window_launches * nwin,
             "serving": serving,
             "batch": batch,
             "density_ratio": var_rho,
@@ -628,7 +645,7 @@ def run_ours(args):
             "small_configs_fp32": small,
             "cpu_baselines": base,
             "square_2048x2048": square,
-            "gpu_launches_half_store": len(HALF_MODES) * args.steps,
+            "gpu_launches_half_store": len(HALF_MODES) * step_launches(args.steps, NX, NY, sms, True),
             "clocks": clocks,
             # last, so that a reader of the line's tail sees them: each 16-bit mode against FP32 at
             # 2048 x 1024, and every storage mode's error against the oracle after 10 000 steps
