@@ -168,18 +168,26 @@ Layout layout_of(const lbm_params* p) {
     return L;
 }
 
-// Step kernel of a new handle: the warp-specialised persistent kernel where it is faster (16-bit
-// storage, and any storage with a density ratio != 1), else the one-tile kernel.
-int default_kernel(int storage, const lbm::Variant& v, int pipe_blocks_per_sm) {
+// Whether a new handle prefers the warp-specialised persistent kernel (if it fits) for single steps: 16-bit
+// storage, and any storage with a density ratio != 1.
+bool prefers_pipelined(int storage, const lbm::Variant& v) {
     // Measured on GB300 (us per step, one-tile / warp-specialised), sheared drop 2048 x 1024: FP32
     // 72.8 / 73.7 (HBM-bound either way); two cells per thread in 32 x 8 tiles: FP16 51.5 / 50.6,
     // BF16 52.0 / 50.7, FP16_FG 55.8 / 54.9, BF16_FG 55.9 / 54.9 (one-tile kernel: five CTAs per
     // SM; warp-specialised: four CTAs of four compute warps and a copy warp, which stages one tile
     // ahead); prescribed velocity, the same grid: FP32 52.5 / 55.1, FP16 40.1 / 37.5; rising bubble
     // 1024 x 2048 (density ratio 10): FP32 81.0 / 80.1, FP16 62.6 / 57.9.
-    if (pipe_blocks_per_sm < 1) return LBM_KERNEL_TILE;
-    if (v.var_rho || storage != LBM_STORE_FP32) return LBM_KERNEL_PIPELINED;
-    return LBM_KERNEL_TILE;
+    return v.var_rho || storage != LBM_STORE_FP32;
+}
+
+// Prepare the warp-specialised kernel of a handle (once) and size its grid; 0 CTAs if it does not fit.
+int prepare_pipelined(lbm_handle* h) {
+    if (h->pipe_ctas >= 0) return LBM_OK;
+    int bps = 0, bps_pipe = 0;
+    const int rc = prepare_kernels(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0), &bps, &bps_pipe);
+    if (rc) return rc;
+    h->pipe_ctas = (int)std::min<long long>((long long)h->tiles_x * h->tiles_y, (long long)bps_pipe * h->sms);
+    return LBM_OK;
 }
 
 lbm::Phys make_phys(const lbm_params* p, const Layout& L) {
@@ -567,14 +575,22 @@ int lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_
     h->tile_ctr = h->status + 2;
     h->last_pipe_step = -2;
     h->partials = reinterpret_cast<double*>(h->ws + L.off_partials);
-    int bps = 0, bps_pipe = 0;
-    rc = prepare_kernels(p->storage, variant_of(*p, h->phys.var_rho != 0), &bps, &bps_pipe);
+    const lbm::TileDims td = lbm::tile_dims(p->storage);
+    h->tiles_x = (p->nx + td.tx - 1) / td.tx;
+    h->tiles_y = (p->ny + td.ty - 1) / td.ty;
+    h->pipe_ctas = -1;
+    int bps = 0;
+    rc = prepare_kernels(p->storage, variant_of(*p, h->phys.var_rho != 0), &bps, nullptr);
     if (!rc && lbm::prepare_run(p->storage, variant_of(*p, h->phys.var_rho != 0), &h->run) != cudaSuccess)
         rc = fail(LBM_ECUDA, "kernel setup failed");
     if (!rc && cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess)
         rc = fail(LBM_ECUDA, "cudaDeviceGetAttribute failed");
+    h->kernel = LBM_KERNEL_TILE;
+    if (!rc && prefers_pipelined(p->storage, variant_of(*p, h->phys.var_rho != 0))) {
+        rc = prepare_pipelined(h);
+        if (h->pipe_ctas > 0) h->kernel = LBM_KERNEL_PIPELINED;
+    }
     const bool pair16 = lbm::pair_is_16bit(p->storage), h16 = lbm::h_is_16bit(p->storage);
-    const lbm::TileDims td = lbm::tile_dims(p->storage);
     const int es_pair = pair16 ? 4 : 8;
     // h boxes: one plane per pair of links (elements of two values: 4 bytes for 16-bit h, 8 for
     // FP32 h), TY + 1 rows to cover both links' source rows
@@ -596,13 +612,6 @@ int lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_
     if (rc) {
         delete h;
         return rc;
-    }
-    h->tiles_x = (p->nx + td.tx - 1) / td.tx;
-    h->tiles_y = (p->ny + td.ty - 1) / td.ty;
-    {
-        const long long ntiles = (long long)h->tiles_x * h->tiles_y, slots = (long long)bps_pipe * h->sms;
-        h->pipe_ctas = (int)(ntiles < slots ? ntiles : slots);
-        h->kernel = default_kernel(p->storage, variant_of(*p, h->phys.var_rho != 0), bps_pipe);
     }
     cudaError_t e = cudaMemsetAsync(h->ws, 0, L.total, h->stream);
     if (e != cudaSuccess) {
@@ -839,14 +848,17 @@ int lbm_set_kernel(lbm_handle* h, int variant) {
     g_err.clear();
     if (!h) return fail(LBM_EINVAL, "handle is NULL");
     if (variant == LBM_KERNEL_AUTO) {
-        int bps = 0, bps_pipe = 0;
-        int rc = prepare_kernels(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0), &bps, &bps_pipe);
-        if (rc) return rc;
-        h->kernel = default_kernel(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0), bps_pipe);
+        h->kernel = prefers_pipelined(h->prm.storage, variant_of(h->prm, h->phys.var_rho != 0)) && h->pipe_ctas > 0
+                        ? LBM_KERNEL_PIPELINED
+                        : LBM_KERNEL_TILE;
         h->chosen = 0;
         return LBM_OK;
     }
     if (variant != LBM_KERNEL_TILE && variant != LBM_KERNEL_PIPELINED) return fail(LBM_EINVAL, "bad kernel variant");
+    if (variant == LBM_KERNEL_PIPELINED) {
+        const int rc = prepare_pipelined(h);
+        if (rc) return rc;
+    }
     if (variant == LBM_KERNEL_PIPELINED && h->pipe_ctas < 1)
         return fail(LBM_EINVAL, "the pipelined kernel does not fit on an SM for this storage mode");
     h->kernel = variant;

@@ -55,7 +55,7 @@ struct lbm_handle {
     CUtensorMap tm_hist[2];  // TMA descriptors of the u history buffers
     int tiles_x, tiles_y;    // step-kernel grid: one tile per CTA (lbm::tile_dims of the storage mode)
     int kernel;              // LBM_KERNEL_TILE or LBM_KERNEL_PIPELINED
-    int pipe_ctas;           // CTAs of the pipelined kernel (0: it does not fit)
+    int pipe_ctas;           // CTAs of the pipelined kernel (0: it does not fit, -1: not prepared)
     int chosen;              // 1: lbm_set_kernel chose it, and every step is a launch of it
     int sms;                 // SMs of the device
     lbm::RunDims run;        // the kernel of a run of steps (blocks_per_sm 0: it does not fit)
