@@ -254,19 +254,21 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
     const bool pair16 = lbm::pair_is_16bit(g.st);
     const int want = (int)((pair16 ? kCohortTiles16 : kCohortTiles) * slots * g.run.buffers);
     const lbm::TileDims td = lbm::tile_dims(g.st);
-    size_t at = 0;
-    for (; at < g.members.size() && runs_alone(b, b->members[g.members[at]]); ++at) {  // (largest first)
-        lbm_handle* h = b->members[g.members[at]];
+    for (int k : g.members) {
+        lbm_handle* h = b->members[k];
+        if (!runs_alone(b, h)) continue;
         const int64_t before = h->launches;
         const int rc = lbm_step(h, n);
         if (rc) return rc;
         b->launches += h->launches - before;
     }
-    for (; at < g.members.size(); at += lbm::kRunMembers) {
+    for (size_t at = 0; at < g.members.size();) {
         lbm::RunManyArgs a;
         std::memset(&a, 0, sizeof(a));
         a.descs = b->d_desc;
-        a.members = (int)std::min<size_t>(lbm::kRunMembers, g.members.size() - at);
+        for (; at < g.members.size() && a.members < lbm::kRunMembers; ++at)
+            if (!runs_alone(b, b->members[g.members[at]])) a.m[a.members++].desc = g.members[at];
+        if (a.members == 0) break;
         int64_t total = 0;
         int first = 0, tiles = 0, before = -1;  // members [first, ..) of the cohort at hand and their tiles; the cohort before
         auto close = [&](int from, int to) {
@@ -280,13 +282,11 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
             for (int k = from; k < to; ++k) a.m[k].tiles = sum;
         };
         for (int k = 0; k < a.members; ++k) {
-            const int idx = g.members[at + k];
-            const lbm_handle* h = b->members[idx];
             lbm::RunMember& m = a.m[k];
+            const lbm_handle* h = b->members[m.desc];
             // (a periodic last tile row of one cell row makes two tile rows of a tile's reach, see lbm_step)
             const int reach = !g.walls && h->prm.ny % td.ty == 1 ? 2 : 1;
             m.rows = reinterpret_cast<unsigned*>(h->partials) + kRowOffset;
-            m.desc = idx;
             m.ntx = (unsigned short)h->tiles_x;
             m.nty = (unsigned short)h->tiles_y;
             m.flags = reach << 2;

@@ -36,10 +36,13 @@ def lattice(stream, flow, nx, ny, storage, k):
     return g
 
 
-def check(torch, sizes, steps, checked, flow, storage):
-    """Batch the lattices for two calls of `steps` steps; the checked members against one-tile launches."""
+def check(torch, sizes, steps, checked, flow, storage, chosen=()):
+    """Batch the lattices for calls of `steps` and 8 steps; the checked members against one-tile launches.
+    The chosen members have the one-tile kernel set for their own steps."""
     stream = torch.cuda.Stream()
     lats = [lattice(stream, flow, nx, ny, storage, k) for k, (nx, ny) in enumerate(sizes)]
+    for k in chosen:
+        lats[k].kernel = "tile"
     b = lbm.Batch(lats, stream)
     b.step(steps)
     b.step(8)
@@ -68,6 +71,11 @@ def test_cohorts_and_member_chunks(torch, flow, storage):
 def test_alone_together_and_few(torch, storage):
     check(torch, [(1100, 1024), (300, 200), (40, 9)], 9, range(3), "walls", storage)
     check(torch, [(40, 24), (2, 2)], 12, range(2), "periodic", storage)
+
+
+def test_large_member_with_a_chosen_kernel(torch):
+    """It joins the others; a smaller member after it still runs alone."""
+    check(torch, [(1100, 1024), (1000, 1024), (300, 200)], 9, range(3), "walls", "fp32", chosen=(0,))
 
 
 def test_more_steps_than_one_launch(torch):
