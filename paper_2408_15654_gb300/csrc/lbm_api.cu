@@ -382,7 +382,15 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     a.ctr = fixed ? nullptr : c;
     a.rows = c + kRowOffset;
     h->last_pipe_step = -2;
-    cudaError_t e = lbm::launch_run(h->prm.storage, a, variant_of(h->prm, h->phys.var_rho != 0), ctas, h->stream);
+    const lbm::Variant v = variant_of(h->prm, h->phys.var_rho != 0);
+    cudaError_t e = lbm::launch_run(h->prm.storage, a, v, ctas, h->stream);
+    if (fixed && e == cudaErrorCooperativeLaunchTooLarge) {
+        // a stream confined to fewer SMs than the device has (that of a green context) cannot hold all CTAs of
+        // fixed positions at once; claimed positions need no CTA that is not there yet
+        cudaGetLastError();
+        a.ctr = c;
+        e = lbm::launch_run(h->prm.storage, a, v, ctas, h->stream);
+    }
     if (e != cudaSuccess) return fail(LBM_ECUDA, "run launch: %s", cudaGetErrorString(e));
     h->launches++;
     return LBM_OK;
