@@ -297,7 +297,9 @@ int lbm_batch_set_members(lbm_batch* b, lbm_handle* const* members, int n);
 int lbm_batch_set_schedule(lbm_batch* b, int schedule, int graph_steps);
 
 /* Advance every member by n steps (asynchronous, like lbm_step).  Each member's device status
- * word collects its own instability flags; read it with lbm_status(member). */
+ * word collects its own instability flags; read it with lbm_status(member).  Should a launch of a run
+ * fail (LBM_ECUDA), members may have advanced by different numbers of steps: lbm_steps_taken(member)
+ * tells each one's, and its state is that of this count. */
 int lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Time each schedule with 16-step graphs, and the fastest of them without a graph, over about

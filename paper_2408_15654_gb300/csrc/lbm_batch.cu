@@ -233,6 +233,13 @@ bool takes_runs(const lbm_batch* b, int64_t n) {
     return tiles <= 1 << 24;
 }
 
+// A lattice was advanced by n steps.
+void count_steps(lbm_handle* h, int64_t n) {
+    h->steps += n;
+    h->cur = (int)((h->cur + n) & 1);
+    h->first = 0;
+}
+
 // Whether a member's tiles fill the GPU by themselves: it then advances by lbm_step, whose kernel reads
 // its constants as kernel parameters.  16-bit storage gains from that at 13 tiles per SM (64-lattice mix
 // FP16, from 10 / 14 tiles per SM on: 302 / 310 us per step), FP32 later (364 / 356).
@@ -241,8 +248,9 @@ bool runs_alone(const lbm_batch* b, const lbm_handle* h) {
     return tiles_of(h) >= (int64_t)(lbm::pair_is_16bit(h->prm.storage) ? kAloneTilesPerSm16 : kAloneTilesPerSm) * b->sms;
 }
 
-// n steps of a group as runs.  The large members go one by one; the others, largest first, are cut into
-// cohorts which one launch advances all steps one after the other (see batch_kernel_run).  A cohort
+// n steps of a group as runs, counted launch by launch: should one fail, every member's step count is that of
+// its state.  The large members go one by one; the others, largest first, are cut into cohorts which one
+// launch advances all steps one after the other (see batch_kernel_run).  A cohort
 // must hold more tiles than the CTAs have claimed, or they wait for the level before (FP32 64-lattice
 // mix, 0.8 / 1.2 / 1.6 / 2 / 3 tiles per staged tile: 367 / 361 / 360 / 364 / 373 us per step), and few
 // enough that its state stays in L2.  16-bit storage gains little from L2 and much from never waiting
@@ -310,17 +318,18 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
         if (a.reach > 1) a.batch = std::min(a.batch, 4);  // eight lanes of the lead warp per tile
         a.ctr = b->d_ctr + 2;
         const int64_t most = std::max<int64_t>(64, (1LL << 20) / total);
-        for (int64_t done = 0; done < n; done += a.nsteps) {
-            a.nsteps = (int)std::min(n - done, most);
+        for (int64_t left = n; left > 0; left -= a.nsteps) {
+            a.nsteps = (int)std::min(left, most);
             for (int k = 0; k < a.members; ++k) {
                 const lbm_handle* h = b->members[a.m[k].desc];
-                a.m[k].steps = h->steps + done;
-                a.m[k].flags = (a.m[k].flags & ~3) | (int)((h->cur + done) & 1) | (h->first && done == 0 ? 2 : 0);
+                a.m[k].steps = h->steps;
+                a.m[k].flags = (a.m[k].flags & ~3) | h->cur | (h->first ? 2 : 0);
             }
             cudaError_t e = lbm::launch_batch_run(g.st, a, lbm::Variant{g.walls, g.lang, g.flow, g.var_rho},
                                                   (int)std::min<int64_t>(total, slots), b->stream);
             if (e != cudaSuccess) return fail(LBM_ECUDA, "batch run launch: %s", cudaGetErrorString(e));
             b->launches += 2;
+            for (int k = 0; k < a.members; ++k) count_steps(b->members[a.m[k].desc], a.nsteps);
         }
     }
     return LBM_OK;
@@ -490,12 +499,12 @@ int lbm_batch_step(lbm_batch* b, int64_t n) {
         if (!h->initialized) return fail(LBM_ESTATE, "a member has no state (lbm_init_fields first)");
     int rc = upload_descs(b);
     if (rc) return rc;
-    const bool runs = takes_runs(b, n);
-    if (runs)
+    if (takes_runs(b, n)) {
         for (size_t k = 0; k < b->groups.size() && !rc; ++k) rc = launch_runs(b, b->groups[k], n);
-    if (rc) return rc;
-    int64_t done = runs ? n : 0;
-    if (!runs && b->graph_steps > 0 && n >= b->graph_steps) {
+        return rc;
+    }
+    int64_t done = 0;
+    if (b->graph_steps > 0 && n >= b->graph_steps) {
         if (!b->graph) {
             rc = build_graph(b);
             if (rc) return rc;
@@ -511,12 +520,7 @@ int lbm_batch_step(lbm_batch* b, int64_t n) {
     for (int s = 0; s < rem && !rc; ++s) rc = launch_one(b, s);
     if (!rc && rem > 0) rc = launch_advance(b, rem);
     if (rc) return rc;
-    for (lbm_handle* h : b->members) {
-        if (runs && runs_alone(b, h)) continue;  // lbm_step counted them
-        h->steps += n;
-        h->cur = (int)((h->cur + n) & 1);
-        h->first = 0;
-    }
+    for (lbm_handle* h : b->members) count_steps(h, n);
     return LBM_OK;
 }
 

@@ -44,3 +44,28 @@ def test_other_launch_errors_are_reported(lib, code):
     lib.fail("r", 0, code)
     assert lib.step(h, 20) == lbm.LBM_ECUDA
     assert len(lib.launches()) == 1 and lib.steps(h) == 0
+
+
+def test_a_failed_batch_run_leaves_every_member_with_the_steps_of_its_state(lib):
+    """A member that runs alone, two groups of cohorts; the launch that fails, and what a retry starts from."""
+    big, small, half = params(1100, 1024), params(300, 200), params(200, 200, "fp16")
+    for at, steps in ((0, [30, 0, 0, 0]), (1, [30, 30, 30, 0])):
+        lib.reset()
+        hs = [lib.lattice(p) for p in (big, small, small, half)]
+        b = lib.batch(hs)
+        lib.fail("R", at, 700)
+        assert lib.batch_step(b, 30) == lbm.LBM_ECUDA
+        assert [lib.steps(h) for h in hs] == steps
+        lib.reset()
+        lib.ok(lib.batch_step(b, 30))
+        assert [lib.steps(h) for h in hs] == [s + 30 for s in steps]
+        assert [r["steps"] for r in lib.launches()] == [steps[0], steps[1], steps[3]]
+
+
+def test_a_batch_run_that_fails_after_others_counts_those(lib):
+    hs = [lib.lattice(params(512, 700)) for _ in range(12)]
+    b = lib.batch(hs)
+    lib.fail("R", 1, 700)
+    assert lib.batch_step(b, 200) == lbm.LBM_ECUDA
+    done = lib.launches()[0]["nsteps"]
+    assert 0 < done < 200 and [lib.steps(h) for h in hs] == [done] * 12
