@@ -184,6 +184,12 @@ int lbm_reduce(lbm_handle* h, int what, double* out);
  * launch failed or no timeout was recorded, LBM_EINVAL for a NULL d_word. */
 int lbm_selftest_wait(unsigned* d_word, void* cuda_stream);
 
+/* The same for the waits inside a run of many steps in one launch (lbm_step, lbm_batch_step).  With it on, the
+ * tiles of h wait in the second step of a run for tiles that nobody updates: the run gives up within
+ * seconds, without a fault, and lbm_status(h) returns LBM_ETIMEOUT (in a batch, every lattice of the launch
+ * does).  The state is lost; lbm_init_fields starts anew.  Off in a new handle. */
+int lbm_selftest_stall(lbm_handle* h, int on);
+
 /* The sum of lbm_reduce for callers that cannot allocate device memory.  (This entry point has no
  * counterpart in the paper; it exists for the library's users.)  Some callers may not call
  * cudaMalloc: a plugin inside a host application whose memory manager owns all device memory, code

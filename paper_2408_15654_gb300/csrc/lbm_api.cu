@@ -342,6 +342,7 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     a.reach = h->prm.bc_y == LBM_BC_PERIODIC && h->prm.ny % td.ty == 1 ? 2 : 1;
     const int slots = h->sms * h->run.blocks_per_sm;
     a.ring = h->run.buffers;
+    a.stall = h->stall;
     a.ahead = 16;
     a.depth = 1;
     a.lag = 1;
@@ -438,9 +439,10 @@ int read_status(lbm_handle* h, unsigned* st) {
     return LBM_OK;
 }
 
-// LBM_OK, LBM_ETIMEOUT (a staging copy did not arrive within its bounded wait) or LBM_EUNSTABLE.
+// LBM_OK, LBM_ETIMEOUT (a staging copy, or in a run of steps a neighbouring tile, was not there within its
+// bounded wait) or LBM_EUNSTABLE.
 int status_code(unsigned st) {
-    if (st & lbm::kStatusTimeout) return fail(LBM_ETIMEOUT, "a bounded wait for a tile copy gave up");
+    if (st & lbm::kStatusTimeout) return fail(LBM_ETIMEOUT, "a bounded wait for a tile gave up");
     if (st & lbm::kStatusUnstable) return fail(LBM_EUNSTABLE, "the device flagged an unstable state");
     return LBM_OK;
 }
@@ -767,6 +769,13 @@ int lbm_reduce(lbm_handle* h, int what, double* out) {
     LBM_CUDA(cudaStreamSynchronize(h->stream));
     *out = r.sum;
     return status_code(r.status);
+}
+
+int lbm_selftest_stall(lbm_handle* h, int on) {
+    g_err.clear();
+    if (!h) return fail(LBM_EINVAL, "handle is NULL");
+    h->stall = on ? 1 : 0;
+    return LBM_OK;
 }
 
 int lbm_status(lbm_handle* h) {

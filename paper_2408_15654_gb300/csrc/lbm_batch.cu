@@ -297,7 +297,7 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
             m.rows = reinterpret_cast<unsigned*>(h->partials) + kRowOffset;
             m.ntx = (unsigned short)h->tiles_x;
             m.nty = (unsigned short)h->tiles_y;
-            m.flags = reach << 2;
+            m.flags = reach << 2 | h->stall << 4;
             a.reach = std::max(a.reach, reach);
             tiles += (int)tiles_of(h);
             total += tiles_of(h);

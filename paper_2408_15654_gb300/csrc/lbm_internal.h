@@ -57,6 +57,7 @@ struct lbm_handle {
     int kernel;              // LBM_KERNEL_TILE or LBM_KERNEL_PIPELINED
     int pipe_ctas;           // CTAs of the pipelined kernel (0: it does not fit, -1: not prepared)
     int chosen;              // 1: lbm_set_kernel chose it, and every step is a launch of it
+    int stall;               // 1: runs wait for tiles that nobody updates (lbm_selftest_stall)
     int sms;                 // SMs of the device
     lbm::RunDims run;        // the kernel of a run of steps (blocks_per_sm 0: it does not fit)
     int cur;          // buffer holding the current state

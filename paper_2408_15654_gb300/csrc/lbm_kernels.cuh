@@ -1629,6 +1629,7 @@ struct RunArgs {
     int ring;                 // tile buffers used, 1 .. RunShape::NB
     int ahead;                // tile j waits in the lead warp until tile j - ahead is signalled (>= ring)
     int batch;                // tiles per round of the lead warp, 1 .. 8 (4 with a reach of two)
+    int stall;                // 1: wait for a tile more than a row has (self-test of the waits)
     unsigned* ctr;            // tile counter of this launch (zero at start), or null: fixed positions
     unsigned* rows;           // tiles finished per tile row (zero at start)
 };
@@ -1643,7 +1644,7 @@ struct RunMember {
     int tiles;                  // tiles in a level of its cohort
     unsigned short first, end;  // members of its cohort
     unsigned short ntx, nty;    // its tiles
-    int flags;                  // buffer of the current state | 2 on the first step after initialisation | reach << 2
+    int flags;                  // buffer of the current state | 2 on the first step after initialisation | reach << 2 | stall << 4
 };
 constexpr int kRunMembers = 96;
 struct RunManyArgs {
@@ -1796,7 +1797,9 @@ __device__ __forceinline__ int ld_shared_acquire(const int* p) {
 __device__ __forceinline__ void st_shared_release(int* p, int v) {
     asm volatile("st.release.cta.shared::cta.s32 [%0], %1;\n" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
-constexpr unsigned kRowPollLimit = 1u << 23;  // polls of 0.1 us or more: the wait ends within seconds
+// Limits of a run's waits in global and shared memory: a second or two, like that of a copy (kWaitLimit).
+constexpr unsigned kRowPollLimit = 1u << 21;  // lead warp: 0.1 us of sleep and a round trip to L2 each
+constexpr unsigned kIdlePollLimit = 1u << 23;  // signal warp: some 0.1 us each
 
 // A run of steps by a persistent, warp-specialised grid of one CTA per SM.  Between steps the grid's
 // tiles wait for their neighbours only, through counters in global memory: no launch, no drained
@@ -1922,24 +1925,24 @@ __device__ __forceinline__ void run_body(const Args& a) {
             const unsigned* rows = nullptr;
             unsigned need = 0u;
             if (live) {
-                int ntx, nty, row, col, reach, flags, member = 0;
+                int ntx, nty, row, col, reach, flags, stall, member = 0;
                 long long steps;
                 if constexpr (kMany) {
                     const RunMember& q = a.m[walk.m];
                     member = walk.m;
-                    ntx = q.ntx, nty = q.nty, reach = q.flags >> 2, flags = q.flags & 3;
+                    ntx = q.ntx, nty = q.nty, reach = q.flags >> 2 & 3, flags = q.flags & 3, stall = q.flags >> 4;
                     rows = q.rows;
                     steps = q.steps;
                     row = (walk.i - q.start) / ntx;
                     col = walk.i - q.start - row * ntx;
                     if (!WALLS) row = (int)((row + (long long)walk.level * reach) % nty);
                 } else {
-                    ntx = a.ntx, nty = a.nty, reach = a.reach, flags = a.cur | (a.first ? 2 : 0);
+                    ntx = a.ntx, nty = a.nty, reach = a.reach, flags = a.cur | (a.first ? 2 : 0), stall = a.stall;
                     rows = a.rows;
                     steps = a.steps;
                     row = walk.row, col = walk.col;
                 }
-                need = (unsigned)walk.level * (unsigned)ntx;
+                need = (unsigned)walk.level * (unsigned)(ntx + stall);
                 entry = make_int4(col * G::TX, row * G::TY,
                                   ((flags + walk.level) & 1) | (walk.level == 0 ? flags & 2 : 0) | (kMany ? member << 2 : 0),
                                   Traits<ST>::kPair16 ? (int)step_seed(steps + walk.level) : 0);
@@ -2061,7 +2064,7 @@ __device__ __forceinline__ void run_body(const Args& a) {
                     }
                 }
             } else {
-                if (++idle == kRowPollLimit) {
+                if (++idle == kIdlePollLimit) {
                     if (lane == 0) flag_timeout();
                     return;
                 }
@@ -2079,19 +2082,18 @@ __device__ __forceinline__ void run_body(const Args& a) {
         const int at = g * Sh::DB + (int)(m % Sh::DB);
         unsigned long long* mbar = &full[at];
         const uint32_t parity = m / Sh::DB & 1u;
-        const bool late = !mbar_wait_bounded(mbar, parity);
-        __syncwarp();
-        const int4 e = queue[at];
+        const bool late = __any_sync(0xffffffffu, !mbar_wait_bounded(mbar, parity));
+        int4 e = queue[at];
+        if (late) e.x = e.y = 0;  // it may be written at this moment: the lanes of a warp take one way all the same
         if (e.x < 0) {
-            // the stop mark; the barrier meets the one in step_tile, should another thread's wait have
-            // given up before it saw the mark
-            if (compute_sync_or<G::NT>(1 + g, late)) compute_sync<G::NT>(1 + g);
+            // the stop mark; another warp's wait may have given up before it saw the mark
+            if (compute_sync_or<G::NT>(1 + g, false)) compute_sync<G::NT>(1 + g);
             else if (lane == 0) mbar_arrive(&done[at]);
             return;
         }
         if constexpr (kMany) {
             // a copy that did not come in time: no constants to read, so meet the barriers of step_tile here
-            if (__any_sync(0xffffffffu, late)) {
+            if (late) {
                 if (lane == 0) flag_timeout();
                 compute_sync_or<G::NT>(1 + g, true);
                 if (lane == 0) mbar_wait_bounded(mbar, parity);
