@@ -308,7 +308,7 @@ int launch_step(lbm_handle* h, int mode, double* const out[5]) {
 // 300 x 300: 5.6 us, a run 7.0; 128 x 128: 5.1 / 4.8; 500 x 300: 7.9 / 7.0).
 bool takes_run(const lbm_handle* h, int64_t n) {
     const long long tiles = (long long)h->tiles_x * h->tiles_y;
-    if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || tiles > 1 << 24) return false;
+    if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || tiles > kRunTiles) return false;
     if (n < (tiles > 8 * h->sms ? 4 : 8)) return false;
     return !(lbm::pair_is_16bit(h->prm.storage) && tiles > h->sms && tiles <= 3 * h->sms);
 }
@@ -333,9 +333,7 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     a.ntx = h->tiles_x;
     a.nty = h->tiles_y;
     const long long tiles = (long long)a.ntx * a.nty;
-    // launches of some tens of milliseconds at most, and positions within 32 bits
-    const int64_t most = std::max<int64_t>(64, (1LL << 20) / tiles);
-    *took = a.nsteps = (int)std::min(n, most);
+    *took = a.nsteps = (int)std::min(n, longest_run(tiles));
     // A tile reads two rows of cells above and below; only a last tile row of one cell row, next to the
     // first around a periodic edge, makes that two tile rows.
     const lbm::TileDims td = lbm::tile_dims(h->prm.storage);

@@ -223,14 +223,11 @@ int launch_one(lbm_batch* b, int s) {
 // more than they save.
 bool takes_runs(const lbm_batch* b, int64_t n) {
     if (b->plain || b->kernel != LBM_KERNEL_AUTO || n < 8) return false;
-    int64_t tiles = 0;
-    for (const lbm_handle* h : b->members) {
-        if (h->tiles_y > kRowCounters) return false;
-        tiles += tiles_of(h);
-    }
+    for (const lbm_handle* h : b->members)
+        if (h->tiles_y > kRowCounters || tiles_of(h) > kRunTiles) return false;
     for (const Group& g : b->groups)
         if (g.run.blocks_per_sm < 1) return false;
-    return tiles <= 1 << 24;
+    return true;
 }
 
 // A lattice was advanced by n steps.
@@ -274,10 +271,15 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
         lbm::RunManyArgs a;
         std::memset(&a, 0, sizeof(a));
         a.descs = b->d_desc;
-        for (; at < g.members.size() && a.members < lbm::kRunMembers; ++at)
-            if (!runs_alone(b, b->members[g.members[at]])) a.m[a.members++].desc = g.members[at];
-        if (a.members == 0) break;
         int64_t total = 0;
+        for (; at < g.members.size() && a.members < lbm::kRunMembers; ++at) {
+            const lbm_handle* h = b->members[g.members[at]];
+            if (runs_alone(b, h)) continue;
+            if (a.members && total + tiles_of(h) > kRunTiles) break;
+            total += tiles_of(h);
+            a.m[a.members++].desc = g.members[at];
+        }
+        if (a.members == 0) break;
         int first = 0, tiles = 0, before = -1;  // members [first, ..) of the cohort at hand and their tiles; the cohort before
         auto close = [&](int from, int to) {
             int sum = 0;
@@ -300,7 +302,6 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
             m.flags = reach << 2 | h->stall << 4;
             a.reach = std::max(a.reach, reach);
             tiles += (int)tiles_of(h);
-            total += tiles_of(h);
             if (tiles >= want) {
                 close(first, k + 1);
                 before = first;
@@ -317,7 +318,7 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
         a.batch = total <= 3LL * slots ? 1 : (!pair16 || total <= 10LL * slots ? 2 : (total <= 16LL * slots ? 4 : 8));
         if (a.reach > 1) a.batch = std::min(a.batch, 4);  // eight lanes of the lead warp per tile
         a.ctr = b->d_ctr + 2;
-        const int64_t most = std::max<int64_t>(64, (1LL << 20) / total);
+        const int64_t most = longest_run(total);
         for (int64_t left = n; left > 0; left -= a.nsteps) {
             a.nsteps = (int)std::min(left, most);
             for (int k = 0; k < a.members; ++k) {

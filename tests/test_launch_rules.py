@@ -66,6 +66,39 @@ def test_a_batch_run_that_fails_after_others_counts_those(lib):
     hs = [lib.lattice(params(512, 700)) for _ in range(12)]
     b = lib.batch(hs)
     lib.fail("R", 1, 700)
-    assert lib.batch_step(b, 200) == lbm.LBM_ECUDA
+    assert lib.batch_step(b, 5000) == lbm.LBM_ECUDA
     done = lib.launches()[0]["nsteps"]
-    assert 0 < done < 200 and [lib.steps(h) for h in hs] == [done] * 12
+    assert 0 < done < 5000 and [lib.steps(h) for h in hs] == [done] * 12
+
+
+@pytest.mark.parametrize("nx,ny,storage,n", [(8, 8, "fp16", 10000), (128, 128, "fp32", 20000), (2048, 1024, "fp32", 3000),
+                                             (2048, 1024, "fp16", 1000), (4096, 4096, "fp32", 200), (8192, 16000, "fp16", 50)])
+def test_a_run_ends_within_some_milliseconds(lib, nx, ny, storage, n):
+    """A tile's update takes some 8 ns at most and a step 4 us at least: no launch beyond 40 ms."""
+    h = lib.lattice(params(nx, ny, storage))
+    lib.ok(lib.step(h, n))
+    done = lib.launches()
+    assert any(r["kind"] == "r" for r in done)
+    assert sum(r["nsteps"] for r in done) == n == lib.steps(h)
+    assert all(max(r["nsteps"] * r["tiles"] * 8e-9, r["nsteps"] * 4e-6) < 0.04 for r in done)
+
+
+def test_a_batch_run_ends_within_some_milliseconds(lib):
+    hs = [lib.lattice(params(1000, 768)) for _ in range(96)] + [lib.lattice(params(16640, 16000))]
+    for h in hs[-1:]:
+        lib.ok(lib.lib.lbm_set_kernel(h, lbm.LBM_KERNEL_TILE))  # joins the others instead of running alone
+    for members in (hs[:8], hs):
+        lib.reset()
+        before = [lib.steps(h) for h in members]
+        b = lib.batch(members)
+        lib.ok(lib.batch_step(b, 600))
+        assert [lib.steps(h) for h in members] == [s + 600 for s in before]
+        assert all(max(r["nsteps"] * r["tiles"] * 8e-9, r["nsteps"] * 4e-6) < 0.04 for r in lib.launches())
+
+
+@pytest.mark.parametrize("nx,ny", [(20000, 16000), (2048, 16136)])
+def test_the_largest_grids_go_step_by_step(lib, nx, ny):
+    """More than 2^20 tiles, or more tile rows than there are counters."""
+    h = lib.lattice(params(nx, ny))
+    lib.ok(lib.step(h, 20))
+    assert [r["kind"] for r in lib.launches()] == ["s"] * 20
