@@ -115,7 +115,10 @@ int build_tiles(lbm_batch* b) {
                      [&](int a, int c) { return tiles_of(b->members[a]) > tiles_of(b->members[c]); });
     std::vector<uint2> tiles;
     for (Group& g : groups) {
-        if (lbm::prepare_batch_run(g.st, lbm::Variant{g.walls, g.lang, g.flow, g.var_rho}, &g.run) != cudaSuccess)
+        // a kernel keeps its set-up while the batch has a group that uses it
+        const auto had = std::find_if(b->groups.begin(), b->groups.end(), [&](const Group& o) { return same_group(o, g); });
+        if (had != b->groups.end()) g.run = had->run;
+        else if (lbm::prepare_batch_run(g.st, lbm::Variant{g.walls, g.lang, g.flow, g.var_rho}, &g.run) != cudaSuccess)
             return fail(LBM_ECUDA, "kernel setup failed");
         for (int k : by_size)
             if (same_group(group_of(b->members[k]), g)) g.members.push_back(k);

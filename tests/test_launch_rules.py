@@ -1,4 +1,6 @@
 """Which launches lbm_step and lbm_batch_step make, with a fake CUDA runtime (no GPU)."""
+import ctypes as C
+
 import pytest
 
 from paper_2408_15654_gb300 import lbm
@@ -102,3 +104,16 @@ def test_the_largest_grids_go_step_by_step(lib, nx, ny):
     h = lib.lattice(params(nx, ny))
     lib.ok(lib.step(h, 20))
     assert [r["kind"] for r in lib.launches()] == ["s"] * 20
+
+
+def test_a_batch_sets_a_kernel_up_once(lib):
+    hs = [lib.lattice(params(64, 64)), lib.lattice(params(96, 64)), lib.lattice(params(64, 64, "fp16"))]
+    b = lib.batch(hs)
+    assert lib.prepared("R") == 2
+    arr = (C.c_void_p * 2)(hs[0], hs[2])
+    for _ in range(3):
+        lib.ok(lib.lib.lbm_batch_set_schedule(b, 1, 0))
+        lib.ok(lib.lib.lbm_batch_set_members(b, arr, 2))
+    assert lib.prepared("R") == 2
+    lib.ok(lib.lib.lbm_batch_set_members(b, (C.c_void_p * 1)(lib.lattice(params(64, 64, walls=True))), 1))
+    assert lib.prepared("R") == 3
