@@ -25,6 +25,8 @@ struct Group {
 
 // Runs of steps, see launch_runs.  Tiles per SM from which a lattice fills the GPU by itself.
 constexpr int kAloneTilesPerSm = 20, kAloneTilesPerSm16 = 10;
+// Tile counters of a batch: two of the launches of single steps, used in turn, and that of a run.
+constexpr int kCounters = 3;
 // Tiles of a cohort for every tile that the launch stages at a time.
 constexpr double kCohortTiles = 1.6, kCohortTiles16 = 6.0;
 
@@ -74,7 +76,7 @@ struct lbm_batch {
     int ws_blocks[5];      // resident warp-specialised CTAs per SM of each members' storage mode (0: none)
     int sms;
     int plain;             // 1: every step is a launch per group, as in lbm_batch_autotune
-    unsigned* d_ctr;       // two tile counters, and that of a run
+    unsigned* d_ctr;       // kCounters tile counters
     int ctr_parity;
     int graph_end_parity;
 };
@@ -407,7 +409,7 @@ int lbm_batch_workspace_bytes(int max_members, int64_t max_tiles, size_t* bytes)
     if (max_members < 1 || max_tiles < 1 || !bytes) return fail(LBM_EINVAL, "need max_members >= 1, max_tiles >= 1");
     if (max_members > (1 << 20) || max_tiles > ((int64_t)1 << 32)) return fail(LBM_EINVAL, "batch too large");
     *bytes = align_up((size_t)max_members * sizeof(lbm::InstDesc)) + align_up((size_t)max_tiles * sizeof(uint2)) +
-             align_up(2 * sizeof(unsigned));
+             align_up(kCounters * sizeof(unsigned));
     return LBM_OK;
 }
 
@@ -447,7 +449,7 @@ int lbm_batch_create(int max_members, int64_t max_tiles, void* d_workspace, size
     int dev = 0;
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ctr, 0, 2 * sizeof(unsigned), b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ctr, 0, kCounters * sizeof(unsigned), b->stream);
     if (e == cudaSuccess) e = cudaEventRecord(b->upload_done, b->stream);
     if (e != cudaSuccess) {
         if (b->upload_done) cudaEventDestroy(b->upload_done);
