@@ -36,6 +36,15 @@ int fail(int code, const char* fmt, ...) {
     return code;
 }
 
+int reach_of(const lbm_handle* h) {
+    return h->prm.bc_y == LBM_BC_PERIODIC && h->prm.ny % lbm::tile_dims(h->prm.storage).ty == 1 ? 2 : 1;
+}
+
+bool few_rows(const lbm_handle* h) {
+    const bool few_warps = lbm::pair_is_16bit(h->prm.storage) && h->phys.var_rho != 0;
+    return h->tiles_y <= 2 * reach_of(h) + 1 + few_warps && (int64_t)h->tiles_x * h->tiles_y > 2 * h->sms;
+}
+
 }  // namespace lbm_host
 
 using namespace lbm_host;
@@ -301,16 +310,42 @@ int launch_step(lbm_handle* h, int mode, double* const out[5]) {
     return LBM_OK;
 }
 
-// Whether `n` steps in a row go as runs (one launch for many steps).  Always the faster way but for a
-// few steps, whose launch and counters' reset cost more than they save (at 128 x 128: 4.3 us per step
-// one by one, 4.0 in a run, 5 us once per run), and for 16-bit grids of one to three tiles per SM,
-// where all tiles are resident at once either way and the one-tile kernel hands over faster (FP16
-// 300 x 300: 5.6 us, a run 7.0; 128 x 128: 5.1 / 4.8; 500 x 300: 7.9 / 7.0).
+// Fewest steps that go as a run (0: never), where that is faster than a launch per step.  A launch and its
+// counters' reset cost 4 to 8 us once; a step's gain over its own launch depends on the grid.  Measured on
+// GB300, us per step one by one / in runs of so many steps:
+int64_t fewest_steps(const lbm_handle* h) {
+    const int64_t tiles = (int64_t)h->tiles_x * h->tiles_y;
+    const bool pair16 = lbm::pair_is_16bit(h->prm.storage), flow = h->prm.velocity == LBM_VELOCITY_SOLVED;
+    const bool var_rho = h->phys.var_rho != 0;
+    if (lbm_host::few_rows(h)) return 0;
+    if (pair16) {
+        // One to three tiles per SM: all are resident at once either way and the one-tile kernel hands over
+        // faster (FP16 300 x 300: 5.6, a run 7.0).
+        if (tiles > h->sms && tiles <= 3 * h->sms) return 0;
+        // Few tiles: a step is one tile's latency either way (BF16_FG 64 x 64: 8 steps 5.15 / 5.89, 64 5.15 / 5.18
+        // with a density ratio; 8 4.00 / 4.41, 16 4.00 / 4.06 with a prescribed velocity; FP16 solved 8 5.16 / 5.39).
+        if (tiles < 64) return flow && !var_rho ? 16 : 32;
+    } else if (!var_rho) {
+        // The one-tile kernel's warps start a tile sooner than those of a run are handed it (64 x 64: 64 steps
+        // 3.51 / 4.06; 112 x 112: 12 steps 4.32 / 4.32).  Without h its step is shorter still, and it holds five
+        // tiles per SM at once, a run three (prescribed, 128 x 128: 64 steps 3.40 / 3.46; 300 x 300: 16 4.02 / 4.44,
+        // 64 4.25 / 4.25; 420 x 420: 8 5.61 / 6.20, 16 5.61 / 5.75, 64 5.61 / 5.35).
+        if (tiles < (flow ? 56 : 80)) return 0;
+        if (!flow && tiles > 2 * h->sms && tiles <= 5 * h->sms) return tiles <= 3 * h->sms ? 0 : 16;
+    }
+    // Short steps and those with few warps gain less per step (700 x 700, 13 tiles per SM, 4 steps: FP16 with a
+    // density ratio 17.2 / 19.0, prescribed FP32 11.9 / 12.8; FP32 sheared drop 700 x 600 16.2 / 14.8).
+    const bool less = !flow || (pair16 && var_rho);
+    if (tiles > (less ? 16 : 8) * h->sms) return 4;
+    return flow || tiles <= 2 * h->sms ? 8 : 12;
+}
+
+// Whether `n` steps in a row go as runs (one launch for many steps).
 bool takes_run(const lbm_handle* h, int64_t n) {
-    const long long tiles = (long long)h->tiles_x * h->tiles_y;
-    if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || tiles > kRunTiles) return false;
-    if (n < (tiles > 8 * h->sms ? 4 : 8)) return false;
-    return !(lbm::pair_is_16bit(h->prm.storage) && tiles > h->sms && tiles <= 3 * h->sms);
+    if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || (int64_t)h->tiles_x * h->tiles_y > kRunTiles)
+        return false;
+    const int64_t fewest = fewest_steps(h);
+    return fewest > 0 && n >= fewest;
 }
 
 // Launch a run of at most n steps; *took receives their number.
@@ -334,10 +369,8 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     a.nty = h->tiles_y;
     const long long tiles = (long long)a.ntx * a.nty;
     *took = a.nsteps = (int)std::min(n, longest_run(tiles));
-    // A tile reads two rows of cells above and below; only a last tile row of one cell row, next to the
-    // first around a periodic edge, makes that two tile rows.
     const lbm::TileDims td = lbm::tile_dims(h->prm.storage);
-    a.reach = h->prm.bc_y == LBM_BC_PERIODIC && h->prm.ny % td.ty == 1 ? 2 : 1;
+    a.reach = lbm_host::reach_of(h);
     const int slots = h->sms * h->run.blocks_per_sm;
     a.ring = h->run.buffers;
     a.stall = h->stall;

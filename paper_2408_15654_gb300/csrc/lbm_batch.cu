@@ -23,8 +23,7 @@ struct Group {
     std::vector<int> members;  // largest first
 };
 
-// Runs of steps, see launch_runs.  Tiles per SM from which a lattice fills the GPU by itself.
-constexpr int kAloneTilesPerSm = 20, kAloneTilesPerSm16 = 10;
+// Runs of steps, see launch_runs.
 // Tile counters of a batch: two of the launches of single steps, used in turn, and that of a run.
 constexpr int kCounters = 3;
 // Tiles of a cohort for every tile that the launch stages at a time.
@@ -224,12 +223,18 @@ int launch_one(lbm_batch* b, int s) {
     return LBM_OK;
 }
 
-// Whether `n` steps go as runs: always the faster way but for a few steps, whose launch and counters cost
-// more than they save.
+// Whether `n` steps go as runs: always the faster way but for lattices of few tile rows and for few steps,
+// whose launch and counters cost more than they save.  With few tiles in all it takes more steps, above all to
+// beat a graph of launches (us per step launches, graph of 16 / runs of 16, of 64 steps: FP32 two lattices
+// 32 x 32 5.0, 4.7 / 5.3, 4.8; two 96 x 96 5.5, 4.8 / 5.0, 4.5).
 bool takes_runs(const lbm_batch* b, int64_t n) {
     if (b->plain || b->kernel != LBM_KERNEL_AUTO || n < 8) return false;
-    for (const lbm_handle* h : b->members)
-        if (h->tiles_y > kRowCounters || tiles_of(h) > kRunTiles) return false;
+    int64_t tiles = 0;
+    for (const lbm_handle* h : b->members) {
+        if (h->tiles_y > kRowCounters || tiles_of(h) > kRunTiles || few_rows(h)) return false;
+        tiles += tiles_of(h);
+    }
+    if (tiles < 96 && n < (b->graph_steps > 0 && n >= b->graph_steps ? 64 : 16)) return false;
     for (const Group& g : b->groups)
         if (g.run.blocks_per_sm < 1) return false;
     return true;
@@ -247,7 +252,10 @@ void count_steps(lbm_handle* h, int64_t n) {
 // FP16, from 10 / 14 tiles per SM on: 302 / 310 us per step), FP32 later (364 / 356).
 bool runs_alone(const lbm_batch* b, const lbm_handle* h) {
     if (h->chosen) return false;  // lbm_step would launch the chosen kernel for every step
-    return tiles_of(h) >= (int64_t)(lbm::pair_is_16bit(h->prm.storage) ? kAloneTilesPerSm16 : kAloneTilesPerSm) * b->sms;
+    int per_sm = 20;
+    if (lbm::pair_is_16bit(h->prm.storage))
+        per_sm = h->prm.velocity == LBM_VELOCITY_SOLVED && !h->phys.var_rho ? 10 : 16;
+    return tiles_of(h) >= (int64_t)per_sm * b->sms;
 }
 
 // n steps of a group as runs, counted launch by launch: should one fail, every member's step count is that of
@@ -263,7 +271,6 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
     const int slots = b->sms * g.run.blocks_per_sm;
     const bool pair16 = lbm::pair_is_16bit(g.st);
     const int want = (int)((pair16 ? kCohortTiles16 : kCohortTiles) * slots * g.run.buffers);
-    const lbm::TileDims td = lbm::tile_dims(g.st);
     for (int k : g.members) {
         lbm_handle* h = b->members[k];
         if (!runs_alone(b, h)) continue;
@@ -299,8 +306,7 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
         for (int k = 0; k < a.members; ++k) {
             lbm::RunMember& m = a.m[k];
             const lbm_handle* h = b->members[m.desc];
-            // (a periodic last tile row of one cell row makes two tile rows of a tile's reach, see lbm_step)
-            const int reach = !g.walls && h->prm.ny % td.ty == 1 ? 2 : 1;
+            const int reach = reach_of(h);
             m.rows = reinterpret_cast<unsigned*>(h->partials) + kRowOffset;
             m.ntx = (unsigned short)h->tiles_x;
             m.nty = (unsigned short)h->tiles_y;

@@ -117,3 +117,54 @@ def test_a_batch_sets_a_kernel_up_once(lib):
     assert lib.prepared("R") == 2
     lib.ok(lib.lib.lbm_batch_set_members(b, (C.c_void_p * 1)(lib.lattice(params(64, 64, walls=True))), 1))
     assert lib.prepared("R") == 3
+
+
+def path(lib, p, n):
+    lib.reset()
+    lib.ok(lib.step(lib.lattice(p), n))
+    return "".join(r["kind"] for r in lib.launches())
+
+
+FLOWS = {"solved": dict(walls=True), "ratio": dict(walls=True, rhoA=1.0, rhoB=0.1),
+         "prescribed": dict(velocity="prescribed")}
+
+
+@pytest.mark.parametrize("storage,flow,nx,ny,never", [
+    ("fp32", "solved", 64, 64, True), ("fp32", "solved", 128, 128, False),      # few tiles
+    ("fp32", "prescribed", 128, 128, True), ("fp32", "ratio", 64, 64, False),
+    ("fp32", "prescribed", 300, 300, True), ("fp32", "prescribed", 160, 160, False),
+    ("fp16", "solved", 300, 300, True), ("fp16", "solved", 128, 128, False),    # one to three tiles per SM
+    ("fp32", "solved", 100000, 8, True), ("fp16", "ratio", 50000, 32, True),    # few tile rows
+    ("fp16", "solved", 50000, 32, False), ("fp32", "solved", 4000, 8, False)])
+def test_grids_that_are_faster_step_by_step_take_no_runs(lib, storage, flow, nx, ny, never):
+    assert path(lib, params(nx, ny, storage, **FLOWS[flow]), 64) == ("s" * 64 if never else "r")
+
+
+@pytest.mark.parametrize("storage,flow,nx,ny,fewest", [
+    ("fp32", "solved", 1024, 1024, 4), ("fp32", "solved", 300, 300, 8), ("fp32", "prescribed", 620, 620, 12),
+    ("fp32", "prescribed", 420, 420, 16), ("fp16", "solved", 700, 600, 4), ("fp16", "ratio", 700, 600, 8),
+    ("fp16", "ratio", 1024, 1024, 4), ("fp16", "solved", 64, 64, 16), ("bf16_fg", "prescribed", 64, 64, 32)])
+def test_few_steps_of_a_grid_go_one_by_one(lib, storage, flow, nx, ny, fewest):
+    p = params(nx, ny, storage, **FLOWS[flow])
+    assert path(lib, p, fewest - 1) == "s" * (fewest - 1) and path(lib, p, fewest) == "r"
+
+
+def batch_path(lib, members, n, graph_steps=0):
+    b = lib.batch([lib.lattice(p) for p in members])
+    lib.ok(lib.lib.lbm_batch_set_schedule(b, 1, graph_steps))
+    lib.reset()
+    lib.ok(lib.batch_step(b, n))
+    return "".join(r["kind"] for r in lib.launches())
+
+
+def test_batches_that_are_faster_step_by_step_take_no_runs(lib):
+    small, flat = [params(64, 64)] * 4, [params(100000, 8), params(300, 300)]
+    assert batch_path(lib, small, 15) == "b" * 15 and batch_path(lib, small, 16) == "R"
+    assert "R" not in batch_path(lib, small, 48, graph_steps=16) and batch_path(lib, small, 64, graph_steps=16) == "R"
+    assert batch_path(lib, flat, 64) == "b" * 64
+
+
+def test_members_of_half_storage_run_alone_from_their_own_size_on(lib):
+    for flow, nx, alone in (("solved", 700, True), ("prescribed", 700, False), ("ratio", 700, False),
+                            ("prescribed", 850, True), ("ratio", 850, True)):
+        assert batch_path(lib, [params(nx, nx, "fp16", **FLOWS[flow])] * 2, 64) == ("rr" if alone else "R")
