@@ -156,9 +156,15 @@ int lbm_init_fields(lbm_handle* h, const double* phi, const double* psi, const d
                     const double* uy, const double* P, int mem);
 
 /* Advance n >= 0 time steps (pull streaming, stencils on halo tiles in shared memory, moment-space
- * collision of f, g and h, fused in one kernel).  Unless lbm_set_kernel chose a kernel, many steps go
- * in one launch, whose tiles wait for their neighbours of the step before (at least 4 or 8 steps,
- * depending on the grid); fewer steps are one launch each.  The state is the same bit for bit.
+ * collision of f, g and h, fused in one kernel).  Unless lbm_set_kernel chose a kernel, steps go as
+ * runs where that is the faster way: many steps in one launch, whose tiles wait for their neighbours
+ * of the step before.  That takes 4 to 32 steps in a row, depending on the grid (8 for most).  One launch
+ * per step remain: fewer steps; FP32 storage at uniform density with fewer than 56 tiles of 32 x 8 cells
+ * (80 with a prescribed velocity, and two to three tiles per SM); 16-bit storage with one to three
+ * tiles per SM; grids of few tile rows (3 to 6, by flow and boundary) with more than two tiles per SM;
+ * more than 2016 tile rows or 2^20 tiles.  A launch takes 4096 steps and 2^22 updates of a tile at most.
+ * The state is the same bit for bit.  While a run is under way, its CTAs hold their SMs (some 35 ms at
+ * most), and its launch waits until all SMs that it needs are free.
  * Asynchronous: errors found by the device surface at the next synchronous call. */
 int lbm_step(lbm_handle* h, int64_t n);
 
@@ -265,8 +271,9 @@ const char* lbm_last_error(void);
  * Not in the paper, which treats one lattice at a time: a batch advances many independent
  * lattices (lbm_handle members, each with its own parameters, grid and workspace), by group of
  * members that share storage mode, boundary kind and EOS: a run of many steps of a group in one
- * launch, or one launch per step and group (see lbm_batch_set_kernel).  Every member's result is bit for bit the one lbm_step gives it alone: a cell's update
- * depends only on its lattice's buffers, constants and step count, never on the schedule.
+ * launch, or one launch per step and group (see lbm_batch_set_kernel).  Every member's result is bit for
+ * bit the one lbm_step gives it alone: a cell's update depends only on its lattice's buffers, constants
+ * and step count, never on the schedule.
  * Ownership: the caller owns the batch workspace and the members; members stay valid and are
  * not destroyed while they belong to a batch (lbm_batch_set_members replaces the list).  All
  * members are created on the batch's stream.  Between batch calls a member may be used through
@@ -286,7 +293,7 @@ int lbm_batch_tiles(lbm_handle* const* members, int n, int64_t* tiles);
 
 /* Device workspace of a batch of up to max_members lattices with up to max_tiles tiles in total:
  * one descriptor per member (TMA maps, constants, buffer pointers, step count), the tile list and
- * the two tile counters of the warp-specialised kernel, each 256-byte aligned. */
+ * the three tile counters of the persistent kernels, each 256-byte aligned. */
 int lbm_batch_workspace_bytes(int max_members, int64_t max_tiles, size_t* bytes);
 
 /* Create an empty batch enqueuing its work on cuda_stream.  CUDA graphs (lbm_batch_set_schedule)
@@ -299,7 +306,9 @@ int lbm_batch_create(int max_members, int64_t max_tiles, void* d_workspace, size
 int lbm_batch_set_members(lbm_batch* b, lbm_handle* const* members, int n);
 
 /* Order of the tiles (LBM_SCHED_*) and the number of steps per captured CUDA graph (0: plain
- * launches) where a step is a launch per group (see lbm_batch_set_kernel).  Default: LBM_SCHED_LARGEST_FIRST, no graph. */
+ * launches) where a step is a launch per group.  Default: LBM_SCHED_LARGEST_FIRST, no graph.  Calls that go as
+ * runs (most calls of eight steps or more under LBM_KERNEL_AUTO) use neither: their tiles come in the
+ * order that runs need.  With LBM_KERNEL_PIPELINED or LBM_KERNEL_TILE set, every call uses both. */
 int lbm_batch_set_schedule(lbm_batch* b, int schedule, int graph_steps);
 
 /* Advance every member by n steps (asynchronous, like lbm_step).  Each member's device status
@@ -309,7 +318,8 @@ int lbm_batch_set_schedule(lbm_batch* b, int schedule, int graph_steps);
 int lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Time each schedule with 16-step graphs, and the fastest of them without a graph, over about
- * trial_steps steps each, one launch per step and group, and keep the fastest.  The trials are real steps: every member
+ * trial_steps steps each, one launch per step and group, and keep the fastest, for the calls that use a
+ * schedule (see lbm_batch_set_schedule); runs are not timed.  The trials are real steps: every member
  * advances by 4 * (16 + trial_steps rounded up to a multiple of 16) + 1 + trial_steps steps
  * (without graphs, on the legacy default stream: 4 * (1 + trial_steps)).  Synchronous. */
 int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_steps);
@@ -319,10 +329,14 @@ int lbm_batch_autotune(lbm_batch* b, int trial_steps, int* schedule, int* graph_
  *   LBM_KERNEL_PIPELINED  persistent, warp-specialised CTAs: a copy warp claims tiles from a
  *                         counter in the workspace and stages each tile's boxes and its lattice's
  *                         constants while the compute warps work on the previous tile;
- *   LBM_KERNEL_AUTO       the default: PIPELINED for calls of fewer than eight steps; from eight
- *                         steps on, runs of many steps in one launch, members of ten tiles per SM or
- *                         more one by one as lbm_step does them, the others together.  Batches of
- *                         16-bit lattices with one to three tiles per SM in all keep PIPELINED.
+ *   LBM_KERNEL_AUTO       the default: from eight steps on, runs of many steps in one launch; the
+ *                         largest members one by one as lbm_step does them (20 tiles per SM or more; 16-bit
+ *                         storage 10, 16 with a density ratio or a prescribed velocity; not those for
+ *                         which lbm_set_kernel chose a kernel), the others together.  PIPELINED for
+ *                         calls of fewer steps, for fewer than 16 steps (64, if the call would use a graph)
+ *                         of batches of fewer than 96 tiles in all, and for batches with a member of few
+ *                         tile rows and more than two tiles per SM, or of more than 2016 tile rows or
+ *                         2^20 tiles.
  * PIPELINED applies only if it fits (else TILE).  lbm_batch_get_kernel reports the setting. */
 int lbm_batch_set_kernel(lbm_batch* b, int variant);
 int lbm_batch_get_kernel(const lbm_batch* b, int* variant);
