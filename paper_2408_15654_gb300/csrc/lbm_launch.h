@@ -96,8 +96,9 @@ cudaError_t launch_step_impl(const StepArgs& a, int mode, const Variant& v, dim3
 }
 
 // A run of steps on `ctas` CTAs, at most one per SM.  With fixed positions (no tile counter) every CTA
-// needs every other, so the launch is cooperative; it follows the counters' reset, so there is no
-// launch before it to overlap with.
+// needs every other, so the launch is cooperative: none of its CTAs starts before all find room (another
+// kernel on 1, 64 or 151 SMs kept all waiting), so none spends its bounded waits on a CTA that has not begun.  It
+// follows the counters' reset, so there is no launch before it to overlap with.
 template <int ST>
 cudaError_t launch_run_impl(const RunArgs& a, const Variant& v, int ctas, cudaStream_t stream) {
     cudaLaunchAttribute attr[1];
