@@ -241,6 +241,10 @@ int lbm_set_state(lbm_handle* h, const void* host_blob, size_t bytes);
 /* Number of steps taken since lbm_init_fields (or restored by lbm_set_state). */
 int lbm_steps_taken(const lbm_handle* h, int64_t* steps);
 
+/* Step kernels launched so far for this lattice alone (a run of many steps is one; launches of a batch that
+ * it belongs to are counted by lbm_batch_launches, those of members that run alone by both). */
+int lbm_launches(const lbm_handle* h, int64_t* launches);
+
 /* Free the handle (not the workspace).  Waits for the handle's stream.  NULL is allowed. */
 int lbm_destroy(lbm_handle* h);
 

@@ -928,6 +928,13 @@ int lbm_steps_taken(const lbm_handle* h, int64_t* steps) {
     return LBM_OK;
 }
 
+int lbm_launches(const lbm_handle* h, int64_t* launches) {
+    g_err.clear();
+    if (!h || !launches) return fail(LBM_EINVAL, "NULL argument");
+    *launches = h->launches;
+    return LBM_OK;
+}
+
 int lbm_destroy(lbm_handle* h) {
     g_err.clear();
     if (!h) return LBM_OK;

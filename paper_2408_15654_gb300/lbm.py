@@ -35,7 +35,7 @@ FIELDS = ("phi", "psi", "ux", "uy", "P")
 # Symbols declared in include/lbm.h (checked by the tests against the header and the library).
 EXPORTS = ("lbm_workspace_bytes", "lbm_create", "lbm_init_fields", "lbm_step", "lbm_get_moments",
            "lbm_reduce", "lbm_reduce_noalloc", "lbm_status", "lbm_state_bytes", "lbm_get_state", "lbm_set_state",
-           "lbm_steps_taken", "lbm_destroy", "lbm_last_error", "lbm_set_kernel", "lbm_get_kernel", "lbm_batch_tiles", "lbm_batch_workspace_bytes",
+           "lbm_steps_taken", "lbm_launches", "lbm_destroy", "lbm_last_error", "lbm_set_kernel", "lbm_get_kernel", "lbm_batch_tiles", "lbm_batch_workspace_bytes",
            "lbm_batch_create", "lbm_batch_set_members", "lbm_batch_set_schedule", "lbm_batch_step",
            "lbm_batch_autotune", "lbm_batch_launches", "lbm_batch_destroy", "lbm_server_workspace_bytes",
            "lbm_server_create", "lbm_server_submit", "lbm_server_poll", "lbm_server_get_stats",
@@ -102,6 +102,7 @@ def load(path: str | None = None):
         "lbm_get_state": [vp, vp, sz],
         "lbm_set_state": [vp, vp, sz],
         "lbm_steps_taken": [vp, C.POINTER(C.c_int64)],
+        "lbm_launches": [vp, C.POINTER(C.c_int64)],
         "lbm_destroy": [vp],
         "lbm_last_error": [],
         "lbm_set_kernel": [vp, C.c_int],
@@ -247,6 +248,12 @@ def lbm_steps_taken(h: int) -> int:
     return v.value
 
 
+def lbm_launches(h: int) -> int:
+    v = C.c_int64()
+    _check(load().lbm_launches(C.c_void_p(h), C.byref(v)))
+    return v.value
+
+
 def lbm_destroy(h: int):
     _check(load().lbm_destroy(C.c_void_p(h)))
 
@@ -308,6 +315,10 @@ class Lattice:
     @property
     def steps(self) -> int:
         return lbm_steps_taken(self.handle)
+
+    @property
+    def launches(self) -> int:
+        return lbm_launches(self.handle)
 
     @property
     def kernel(self) -> str:

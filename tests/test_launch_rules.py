@@ -168,3 +168,12 @@ def test_members_of_half_storage_run_alone_from_their_own_size_on(lib):
     for flow, nx, alone in (("solved", 700, True), ("prescribed", 700, False), ("ratio", 700, False),
                             ("prescribed", 850, True), ("ratio", 850, True)):
         assert batch_path(lib, [params(nx, nx, "fp16", **FLOWS[flow])] * 2, 64) == ("rr" if alone else "R")
+
+
+def test_launches_are_counted(lib):
+    h, n = lib.lattice(params(128, 128)), C.c_int64()
+    for steps, total in ((5, 5), (20, 6), (9000, 9)):
+        lib.ok(lib.step(h, steps))
+        lib.ok(lib.lib.lbm_launches(h, C.byref(n)))
+        assert n.value == total == len(lib.launches())
+    assert lib.lib.lbm_launches(None, C.byref(n)) == lbm.LBM_EINVAL
