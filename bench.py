@@ -5,15 +5,16 @@
 Workload: the sheared drop on a 2048 x 1024 grid (walls at +/-0.01, R = 160, Re = 1, Ca = 0.2,
 Langmuir EOS E0 = 0.2, psi0 = 0.3), populations stored in FP32, synthetic seeded fields.  A step is
 one fused collide-stream update of the whole grid; a window is one lbm_step(K), which launches a
-persistent kernel for up to 128 steps at a time.  The metric is MLUPS (million lattice updates per second; one update advances f, g and h of one cell).  The
-populations (436 MB) exceed the 129 MB L2, so no flush is needed between steps.
+persistent kernel for up to 512 steps at a time.  The metric is MLUPS (million lattice updates per
+second; one update advances f, g and h of one cell).  The populations (436 MB) exceed the 129 MB L2,
+so no flush is needed between steps.
 
 Timing: after W untimed steps, windows of exactly K steps are timed with CUDA events on the
 lattice's stream, back to back, until at least one second of steps has been timed; the value is
 the median window.  nvidia-smi samples the SM clock and throttle reasons over all timed legs.
 
 Printed (one JSON line on rank 0): the device-timed throughput, the end-to-end throughput through
-the C ABI with host buffers, the roofline of the step kernel against the measured HBM bandwidth,
+the C ABI with host buffers, the roofline of a step against the measured HBM bandwidth,
 the FP64 CPU oracle on the host cores as a baseline (every configuration, all cores and one), the
 other legs (square grid, 16-bit storage, prescribed velocity, density ratio, many lattices,
 serving) and the storage errors against the oracle.  With --gpus N > 1 (under torchrun) every rank
@@ -234,17 +235,9 @@ def timed_windows(torch, stream, advance, k: int, min_s: float = None, max_windo
     return statistics.median(times), len(times)
 
 
-def step_launches(n: int, nx: int, ny: int, sms: int, pair16: bool = False) -> int:
-    """Step kernels that one lbm_step(n) launches: runs of max(64, 2^20 / tiles) steps, and one launch per
-    step for a few steps or for 16-bit grids of one to three tiles per SM."""
-    tiles = -(-nx // 32) * -(-ny // 8)
-    launches = 0
-    while n > 0:
-        runs = n >= (4 if tiles > 8 * sms else 8) and not (pair16 and sms < tiles <= 3 * sms)
-        took = min(n, max(64, (1 << 20) // tiles)) if runs else 1
-        n -= took
-        launches += 1
-    return launches
+def path_of(launches: int, steps: int, kernel: str) -> str:
+    """What did the timed steps: runs of many steps in one launch, or the kernel of single steps."""
+    return "runs" if launches < steps else kernel
 
 
 def oracle_mlups(oracle, p, f, threads: int, budget_s: float, max_steps: int = 200):
@@ -312,7 +305,7 @@ def batch_leg(torch, lbm, W, storage: str, steps: int, alone_steps: int = 0):
         lats.append(g)
     cells = sum(g.nx * g.ny for g in lats)
     b = lbm.Batch(lats, bstream)
-    sched, k = b.autotune(trial_steps=32)
+    sched, k = b.autotune(trial_steps=32)  # of calls that launch every step; runs use neither
     torch.cuda.synchronize()
     n0 = b.launches
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -326,19 +319,19 @@ def batch_leg(torch, lbm, W, storage: str, steps: int, alone_steps: int = 0):
     bpl = BYTES_PER_LUP if storage == "fp32" else HALF_MODES[storage]
     out = {"value": sig(cells * steps / (ms * 1e-3) / 1e6), "unit": "MLUPS", "storage": storage, "steps": steps,
            "ms_per_step": sig(ms / steps), "schedule": sched, "graph_steps": k, "gpu_launches": b.launches - n0,
+           "kernel": path_of(b.launches - n0, steps, "pipelined"),
            "achieved_gbs": sig(cells * bpl * steps / (ms * 1e-3) / 1e9),
            "frac_of_measured_hbm": sig(cells * bpl * steps / (ms * 1e-3) / 1e9 / measured_peak()[0])}
     if alone_steps:
         a0, a1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        n0 = sum(g.launches for g in lats)
         a0.record(bstream)
         for g in lats:
             g.step(alone_steps)
         a1.record(bstream)
         torch.cuda.synchronize()
         out["one_at_a_time"] = {"value": sig(cells * alone_steps / (a0.elapsed_time(a1) * 1e-3) / 1e6),
-                                "unit": "MLUPS", "steps": alone_steps, "gpu_launches": sum(step_launches(alone_steps, g.nx, g.ny,
-                                                                  torch.cuda.get_device_properties(0).multi_processor_count,
-                                                                  storage != "fp32") for g in lats)}
+                                "unit": "MLUPS", "steps": alone_steps, "gpu_launches": sum(g.launches for g in lats) - n0}
     b.close()
     for g in lats:
         g.close()
@@ -392,15 +385,17 @@ def lattice_leg(torch, lbm, p, f, args, stream, world, what: str, bytes_per_lup)
     sim.step(args.warmup)
     torch.cuda.synchronize()
     barrier(world)
+    n0 = sim.launches
     ms, nwin = timed_windows(torch, stream, sim.step, args.steps)
     ms_max = barrier_max(ms, world)
     if sim.status != lbm.LBM_OK:
         raise RuntimeError(f"unstable state in the {what} benchmark: {lbm.lbm_last_error()}")
-    kernel = sim.kernel
+    launches = sim.launches - n0
+    kernel = path_of(launches, args.steps * nwin, sim.kernel)
     sim.close()
     cells = p["nx"] * p["ny"]
     out = {"value": sig(cells * args.steps * world / (ms_max * 1e-3) / 1e6), "unit": "MLUPS",
-           "us_per_step": sig(ms_max / args.steps * 1e3), "windows": nwin, "kernel": kernel}
+           "us_per_step": sig(ms_max / args.steps * 1e3), "windows": nwin, "kernel": kernel, "gpu_launches": launches}
     if bytes_per_lup:
         ach = cells * bytes_per_lup / (ms / args.steps * 1e-3) / 1e9
         out.update({"achieved_gbs": sig(ach), "frac_of_measured_hbm": sig(ach / measured_peak()[0]),
@@ -507,7 +502,9 @@ def run_ours(args):
     torch.cuda.synchronize()
     barrier(world)
     torch.cuda.synchronize()
+    n0 = sim.launches
     ms, nwin = timed_windows(torch, stream, sim.step, args.steps)
+    timed_launches = sim.launches - n0
     torch.cuda.synchronize()
     barrier(world)
     ms_max = barrier_max(ms, world)
@@ -515,15 +512,14 @@ def run_ours(args):
         raise RuntimeError(f"unstable state during the benchmark: {lbm.lbm_last_error()}")
     value = aggregate_mlups(cells, args.steps, world, ms_max)
     timed_steps = args.steps * nwin
-    sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-    window_launches = step_launches(args.steps, NX, NY, sms)
 
     # ---- the same workload with 16-bit population storage (FP32 arithmetic) ----
-    half = {}
+    half, half_launches = {}, 0
     for st, bpl in HALF_MODES.items():
         r = lattice_leg(torch, lbm, dict(p, storage=st), f, args, stream, world, st, bpl)
         half[st] = {"MLUPS": r["value"], "x_fp32": sig(r["value"] / value, 3), "us": r["us_per_step"],
                     "hbm_frac": r["frac_of_measured_hbm"], "B_per_lup": bpl}
+        half_launches += r["gpu_launches"]
 
     # ---- the square 2048 x 2048 grid (the second roofline lattice), FP32 and FP16 ----
     sp, sf = W.shear_drop(NX, NX, R=160.0)
@@ -567,7 +563,8 @@ def run_ours(args):
     # ---- errors of every storage mode against the oracle after 10 000 steps (untimed) ----
     precision = precision_leg(torch, lbm, W, stream) if (rank == 0 and not args.no_precision) else None
 
-    # ---- roofline of the step kernel (one launch per step, so launch duration = step time) ----
+    # ---- roofline of a step: algorithmic bytes per step over its time (in a run, rows are updated several
+    # times while they are in L2, so that more bytes are worked on than HBM moves) ----
     peak, peak_kind = measured_peak()
     launch_s = ms / args.steps * 1e-3
     achieved = cells * BYTES_PER_LUP / launch_s / 1e9
@@ -624,7 +621,8 @@ def run_ours(args):
                        "l2": "inputs larger than L2 (2 x 218 MB population buffers), no flush",
                        "timing": f"median of {nwin} back-to-back windows of {args.steps} steps ({timed_steps} steps)"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": traffic,
+                         "frac": achieved / peak, "traffic": traffic, "kernel": path_of(timed_launches, timed_steps, "tile"),
+                         "note": "algorithmic bytes; in a run, rows are updated several times while they are in L2",
                          "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
                          "algorithmic_bytes_per_lup": BYTES_PER_LUP,
                          "survey_bytes_per_lup": BYTES_PER_LUP_SURVEY,
@@ -637,7 +635,7 @@ def run_ours(args):
             "e2e": {"value": e2e, "unit": "MLUPS", "h2d_bytes_per_step": io_bytes / args.steps,
                     "d2h_bytes_per_step": io_bytes / args.steps,
                     "job": f"lbm_init_fields(host) + lbm_step({args.steps}) + lbm_get_moments(host, all 5)"},
-            "gpu_launches": window_launches * nwin,
+            "gpu_launches": timed_launches,
             "serving": serving,
             "batch": batch,
             "density_ratio": var_rho,
@@ -645,7 +643,7 @@ def run_ours(args):
             "small_configs_fp32": small,
             "cpu_baselines": base,
             "square_2048x2048": square,
-            "gpu_launches_half_store": len(HALF_MODES) * step_launches(args.steps, NX, NY, sms, True),
+            "gpu_launches_half_store": half_launches,
             "clocks": clocks,
             # last, so that a reader of the line's tail sees them: each 16-bit mode against FP32 at
             # 2048 x 1024, and every storage mode's error against the oracle after 10 000 steps
