@@ -161,7 +161,8 @@ int lbm_init_fields(lbm_handle* h, const double* phi, const double* psi, const d
  * of the step before.  That takes 4 to 32 steps in a row, depending on the grid (8 for most).  One launch
  * per step remain: fewer steps; FP32 storage at uniform density with fewer than 56 tiles of 32 x 8 cells
  * (80 with a prescribed velocity, and two to three tiles per SM); 16-bit storage with one to three
- * tiles per SM; grids of few tile rows (3 to 6, by flow and boundary) with more than two tiles per SM;
+ * tiles per SM, or narrow (3 to 12 tiles, by flow and size); grids of three tile rows or fewer (four
+ * for 16-bit storage with a density ratio) with more than two tiles per SM;
  * more than 2016 tile rows or 2^20 tiles.  A launch takes 4096 steps and 2^22 updates of a tile at most.
  * The state is the same bit for bit.  While a run is under way, its CTAs hold their SMs (some 35 ms at
  * most), and its launch waits until all SMs that it needs are free.

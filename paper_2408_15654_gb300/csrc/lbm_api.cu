@@ -42,7 +42,7 @@ int reach_of(const lbm_handle* h) {
 
 bool few_rows(const lbm_handle* h) {
     const bool few_warps = lbm::pair_is_16bit(h->prm.storage) && h->phys.var_rho != 0;
-    return h->tiles_y <= 2 * reach_of(h) + 1 + few_warps && (int64_t)h->tiles_x * h->tiles_y > 2 * h->sms;
+    return h->tiles_y <= 3 + few_warps && (int64_t)h->tiles_x * h->tiles_y > 2 * h->sms;
 }
 
 }  // namespace lbm_host
@@ -325,28 +325,40 @@ int64_t fewest_steps(const lbm_handle* h) {
         // Few tiles: a step is one tile's latency either way (BF16_FG 64 x 64: 8 steps 5.15 / 5.89, 64 5.15 / 5.18
         // with a density ratio; 8 4.00 / 4.41, 16 4.00 / 4.06 with a prescribed velocity; FP16 solved 8 5.16 / 5.39).
         if (tiles < 64) return flow && !var_rho ? 16 : 32;
+        // Narrow grids: the tiles at the sides take longer, and a run's positions and claims give them to the same
+        // CTAs in every row, where launches hand out tile by tile (four tiles wide, 16 steps, 5.5 / 12.5 tiles per
+        // SM, run / launches: FP16 periodic 1.10 / 1.14, density ratio 1.17 / 1.17, between walls 0.97 / 1.03; six wide
+        // 1.11 / 1.10, 1.13 / 1.16, 0.95 / 1.00; eight wide 0.82 / 1.07, 0.90 / 1.13, 0.79 / 0.99; twelve wide at 50 per SM
+        // 1.18, 1.12, 1.05; prescribed, six wide, 5.5 / 16 / 25 per SM 0.87 / 1.15 / 0.91).
+        const bool many = tiles > 10 * h->sms, uneven = var_rho || h->prm.bc_y == LBM_BC_PERIODIC;
+        if (flow && (uneven || many) && h->tiles_x >= 3 && h->tiles_x <= (!many ? 6 : uneven ? 12 : 8)) return 0;
+        if (!flow && many && tiles <= 20 * h->sms && h->tiles_x >= 3 && h->tiles_x <= 6) return 0;
     } else if (!var_rho) {
         // The one-tile kernel's warps start a tile sooner than those of a run are handed it (64 x 64: 64 steps
         // 3.51 / 4.06; 112 x 112: 12 steps 4.32 / 4.32).  Without h its step is shorter still, and it holds five
         // tiles per SM at once, a run three (prescribed, 128 x 128: 64 steps 3.40 / 3.46; 300 x 300: 16 4.02 / 4.44,
-        // 64 4.25 / 4.25; 420 x 420: 8 5.61 / 6.20, 16 5.61 / 5.75, 64 5.61 / 5.35).
+        // 64 4.0 / 4.2; 360 x 360: 8 6.0 / 5.6; 420 x 420: 8 5.6 / 6.2, 16 5.6 / 5.7, 64 5.6 / 5.3).
         if (tiles < (flow ? 56 : 80)) return 0;
-        if (!flow && tiles > 2 * h->sms && tiles <= 5 * h->sms) return tiles <= 3 * h->sms ? 0 : 16;
+        if (!flow && tiles > 2 * h->sms && tiles <= 3 * h->sms) return 0;
+        if (!flow && tiles > 4 * h->sms && tiles <= 5 * h->sms) return 16;
     }
     // Short steps and those with few warps gain less per step (700 x 700, 13 tiles per SM, 4 steps: FP16 with a
     // density ratio 17.2 / 19.0, prescribed FP32 11.9 / 12.8; FP32 sheared drop 700 x 600 16.2 / 14.8).
     const bool less = !flow || (pair16 && var_rho);
     if (tiles > (less ? 16 : 8) * h->sms) return 4;
-    return flow || tiles <= 2 * h->sms ? 8 : 12;
+    return flow || (tiles > 128 && tiles <= 4 * h->sms) ? 8 : 12;
 }
 
-// Whether `n` steps in a row go as runs (one launch for many steps).
-bool takes_run(const lbm_handle* h, int64_t n) {
+}  // namespace
+
+bool lbm_host::takes_run(const lbm_handle* h, int64_t n) {
     if (h->chosen || h->run.blocks_per_sm < 1 || h->tiles_y > kRowCounters || (int64_t)h->tiles_x * h->tiles_y > kRunTiles)
         return false;
     const int64_t fewest = fewest_steps(h);
     return fewest > 0 && n >= fewest;
 }
+
+namespace {
 
 // Launch a run of at most n steps; *took receives their number.
 int launch_run(lbm_handle* h, int64_t n, int64_t* took) {

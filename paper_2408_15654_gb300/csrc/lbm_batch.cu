@@ -250,8 +250,8 @@ void count_steps(lbm_handle* h, int64_t n) {
 // Whether a member's tiles fill the GPU by themselves: it then advances by lbm_step, whose kernel reads
 // its constants as kernel parameters.  16-bit storage gains from that at 13 tiles per SM (64-lattice mix
 // FP16, from 10 / 14 tiles per SM on: 302 / 310 us per step), FP32 later (364 / 356).
-bool runs_alone(const lbm_batch* b, const lbm_handle* h) {
-    if (h->chosen) return false;  // lbm_step would launch the chosen kernel for every step
+bool runs_alone(const lbm_batch* b, const lbm_handle* h, int64_t n) {
+    if (!takes_run(h, n)) return false;  // lbm_step would launch every step: a chosen kernel, a narrow grid
     int per_sm = 20;
     if (lbm::pair_is_16bit(h->prm.storage))
         per_sm = h->prm.velocity == LBM_VELOCITY_SOLVED && !h->phys.var_rho ? 10 : 16;
@@ -273,7 +273,7 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
     const int want = (int)((pair16 ? kCohortTiles16 : kCohortTiles) * slots * g.run.buffers);
     for (int k : g.members) {
         lbm_handle* h = b->members[k];
-        if (!runs_alone(b, h)) continue;
+        if (!runs_alone(b, h, n)) continue;
         const int64_t before = h->launches;
         const int rc = lbm_step(h, n);
         if (rc) return rc;
@@ -286,7 +286,7 @@ int launch_runs(lbm_batch* b, const Group& g, int64_t n) {
         int64_t total = 0;
         for (; at < g.members.size() && a.members < lbm::kRunMembers; ++at) {
             const lbm_handle* h = b->members[g.members[at]];
-            if (runs_alone(b, h)) continue;
+            if (runs_alone(b, h, n)) continue;
             if (a.members && total + tiles_of(h) > kRunTiles) break;
             total += tiles_of(h);
             a.m[a.members++].desc = g.members[at];

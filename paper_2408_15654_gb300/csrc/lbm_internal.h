@@ -85,7 +85,11 @@ int reach_of(const lbm_handle* h);
 // Whether (nearly) every tile row reads every other, so that in a run each step waits for the whole step before
 // it, and there are more tiles than that leaves room for: one launch per step is then faster (100000 x 8, us per
 // step one by one / 64 steps in a run: FP32 34.6 / 35.9, FP16 25.5 / 28.6, rising bubble 30.7 / 35.2; 4000 x 24
-// prescribed FP32 4.5 / 6.0; 50000 x 32, four rows: rising bubble FP16 49.3 / 51.3, FP16 drop 41.3 / 39.4).
+// prescribed FP32 4.5 / 6.0; 50000 x 32, four rows: rising bubble FP16 49.3 / 51.3, FP16 drop 41.3 / 39.4; five rows
+// with a reach of two, 20000 x 33 and 4000 x 33: FP32 28.9 / 27.8, 7.4 / 7.8; FP16 23.3 / 23.9, 10.5 / 9.2).
 bool few_rows(const lbm_handle* h);
+
+// Whether lbm_step does `n` steps in a row as runs (many steps in one launch).
+bool takes_run(const lbm_handle* h, int64_t n);
 
 }  // namespace lbm_host

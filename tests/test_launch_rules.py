@@ -125,7 +125,7 @@ def path(lib, p, n):
     return "".join(r["kind"] for r in lib.launches())
 
 
-FLOWS = {"solved": dict(walls=True), "ratio": dict(walls=True, rhoA=1.0, rhoB=0.1),
+FLOWS = {"solved": dict(walls=True), "periodic": {}, "ratio": dict(walls=True, rhoA=1.0, rhoB=0.1),
          "prescribed": dict(velocity="prescribed")}
 
 
@@ -135,7 +135,11 @@ FLOWS = {"solved": dict(walls=True), "ratio": dict(walls=True, rhoA=1.0, rhoB=0.
     ("fp32", "prescribed", 300, 300, True), ("fp32", "prescribed", 160, 160, False),
     ("fp16", "solved", 300, 300, True), ("fp16", "solved", 128, 128, False),    # one to three tiles per SM
     ("fp32", "solved", 100000, 8, True), ("fp16", "ratio", 50000, 32, True),    # few tile rows
-    ("fp16", "solved", 50000, 32, False), ("fp32", "solved", 4000, 8, False)])
+    ("fp16", "solved", 50000, 32, False), ("fp32", "solved", 4000, 8, False), ("fp16", "periodic", 4000, 33, False),
+    ("fp16", "periodic", 120, 1600, True), ("fp16", "periodic", 250, 800, False),           # narrow
+    ("bf16_fg", "ratio", 180, 1100, True), ("fp16", "solved", 120, 1600, False), ("fp16", "solved", 250, 2000, True),
+    ("fp16", "solved", 280, 2000, False), ("fp32", "periodic", 120, 1600, False),
+    ("fp16", "prescribed", 120, 1600, False)])
 def test_grids_that_are_faster_step_by_step_take_no_runs(lib, storage, flow, nx, ny, never):
     assert path(lib, params(nx, ny, storage, **FLOWS[flow]), 64) == ("s" * 64 if never else "r")
 
@@ -177,3 +181,8 @@ def test_launches_are_counted(lib):
         lib.ok(lib.lib.lbm_launches(h, C.byref(n)))
         assert n.value == total == len(lib.launches())
     assert lib.lib.lbm_launches(None, C.byref(n)) == lbm.LBM_EINVAL
+
+
+def test_a_narrow_member_joins_the_others(lib):
+    narrow = params(250, 4000, "fp16")
+    assert path(lib, narrow, 64) == "s" * 64 and batch_path(lib, [narrow] * 2, 64) == "R"
