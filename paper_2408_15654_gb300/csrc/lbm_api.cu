@@ -393,9 +393,9 @@ int launch_run(lbm_handle* h, int64_t n, int64_t* took) {
     // Updating a row several times while it is in L2 pays for FP32 storage beyond L2 (129 MB), whose
     // step is bound by HBM, where the rows in flight leave room for it: `lag` rows between levels must
     // hold twice the tiles staged at a time, or tiles wait for the level before, and the band of
-    // depth x lag rows has to stay in L2 (us per step, one level at a time / so: sheared drop
-    // 2048 x 1024 68.8 / 67.1, 2048^2 136.5 / 132.5, rising bubble 1024 x 2048 76.7 / 72.8; FP16
-    // sheared drop 43.3 / 49.0).
+    // depth x lag rows has to stay in L2 (104 MB of its 129; 160 MB: both buffers of a state well beyond
+    // it).  us per step, one level at a time / so: sheared drop 2048 x 1024 68.8 / 67.1, 2048^2
+    // 136.5 / 132.5, rising bubble 1024 x 2048 76.7 / 72.8; FP16 sheared drop 43.3 / 49.0.
     const double cell_bytes = 2.0 * (lbm::pop_bytes_per_cell(h->prm.storage, h->prm.velocity == LBM_VELOCITY_SOLVED) +
                                      sizeof(float2) * (h->shist[0] ? 2 : 1));
     const double row_bytes = cell_bytes * h->L.pitch * td.ty;

@@ -1,6 +1,6 @@
 // Many independent lattices advanced together, by group of lattices that share a storage mode,
-// boundary kind and EOS.  Eight steps or more go as runs, one launch per group for many steps
-// (launch_runs).  Fewer, or with a kernel chosen by lbm_batch_set_kernel: one launch of the many-lattice
+// boundary kind and EOS.  Most calls of eight steps or more go as runs, one launch per group for many steps
+// (takes_runs, launch_runs).  Others, or with a kernel chosen by lbm_batch_set_kernel: one launch of the many-lattice
 // kernel per step and group, over the group's tile list, whose order is the schedule; graph_steps
 // such steps are captured once into a CUDA graph and replayed.  The workspace holds a descriptor
 // per lattice (TMA maps, constants, buffers, step count) and the tile lists.

@@ -1807,7 +1807,7 @@ constexpr unsigned kIdlePollLimit = 1u << 23;  // signal warp: some 0.1 us each
 // while it is in L2.  Sheared drop, us per step, one launch per step / a run: FP32 128 x 128 4.3 / 4.0,
 // 512 x 256 6.6 / 5.5, 608 x 512 10.4 / 8.3, 2048 x 1024 73.2 / 67.1 (one level at a time 68.8, which
 // is the measured copy rate); FP16 1024 x 512 14.7 / 12.4, 2048 x 1024 50.3 / 43.3; BF16_FG
-// 1531 x 787 35.6 / 28.4.  One group of CTAs per tile and step left the SM idle between a tile's
+// 1531 x 787 35.6 / 28.4.  Which grids take runs is decided on the host (fewest_steps).  One group of CTAs per tile and step left the SM idle between a tile's
 // copy and its arithmetic; here three groups (FP32; four of half the threads with two cells per
 // thread) have their next tiles in shared memory.
 // What bounds it: FP32 storage HBM and L2 latency (five buffers of 41 KB fill the SM), 16-bit storage
@@ -2127,13 +2127,17 @@ __device__ __forceinline__ void run_body(const Args& a) {
     }
 }
 
+// Registers: the launch shape gives every thread of a CTA the same number, the four support warps as many as
+// the compute warps (FP32 72, with a density ratio 92; 16-bit 96 in four groups, with a density ratio 128 in three).
+// 16-bit storage with a density ratio between walls spills 8 to 16 bytes of its 128.
 template <int ST, bool WALLS, bool LANGMUIR, int FLOW>
 __global__ void __launch_bounds__(RunShape<ST, FLOW>::THREADS, 1) step_kernel_run(const __grid_constant__ RunArgs a) {
     run_body<ST, WALLS, LANGMUIR, FLOW>(a);
 }
 // The same for many lattices.  A tile's lattice constants come with its boxes (one more bulk copy), which
 // costs registers: with two cells per thread three groups of 128 registers do better than four of 96,
-// which spill (64-lattice mix FP16: 321 / 366 us per step).  What bounds it: with FP32 storage and
+// which spill (64-lattice mix FP16: 321 / 366 us per step); FP32 storage between walls spills 8 bytes of 72.
+// What bounds it: with FP32 storage and
 // the state in L2 the compute groups wait for tiles 40 % of the time and issue in 48 % of the cycles (five
 // buffers fill the SM: with four the mix takes 414 us instead of 373), with 16-bit storage the latency
 // of the cell update at twelve compute warps per SM.
